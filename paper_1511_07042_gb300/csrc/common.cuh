@@ -330,8 +330,9 @@ constexpr double kDropFP32 = 1e-5;
 // sel_first < 0: the k pairs of smallest |theta| (index-updating); >= 0: positions
 // sel_first .. sel_first + k - 1 of the ascending values (index-fixed; moved down when
 // past the top), ordered by (|theta|, theta, index) like the former.
+// salt: set of start vectors of the inverse iteration (another one for a second attempt).
 void dense_eig(const double* Ahat, const double* Mhat, int n, double sigma, int k,
                double* theta, double* Y, int* rank, double* work, double* quality, double drop_tol,
-               int nq, cudaStream_t s, int sel_first = -1);
+               int nq, cudaStream_t s, int sel_first = -1, int salt = 0);
 size_t dense_work_doubles(int n);
 }  // namespace bmg

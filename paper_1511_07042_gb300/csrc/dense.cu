@@ -623,8 +623,9 @@ trsm_kernel(const double* __restrict__ Ahat, const double* __restrict__ Mhat, in
 // from an integer hash of (row, column).  Vectors with a common positive component
 // project almost parallel onto a near-degenerate group, and the last member of the
 // group then keeps almost nothing after orthogonalisation.
-__device__ __forceinline__ float start_value(int a, int j) {
-  unsigned x = ((unsigned)a * 0x9E3779B1u) ^ ((unsigned)(j + 1) * 0x85EBCA77u);
+// salt: another set of values (0: the first attempt's).
+__device__ __forceinline__ float start_value(int a, int j, unsigned salt) {
+  unsigned x = ((unsigned)a * 0x9E3779B1u) ^ ((unsigned)(j + 1) * 0x85EBCA77u) ^ (salt * 0xC2B2AE3Du);
   x ^= x >> 15;
   x *= 0x2C1B3C6Du;
   x ^= x >> 12;
@@ -904,7 +905,7 @@ constexpr int kInvThreads = 64;
 constexpr int kInvSmemMembers = 63;
 constexpr int kInvLuFloats = 24 * 1024;   // shared memory for the LU factors (96 KB)
 __global__ void __launch_bounds__(kInvThreads)
-invit_kernel(int n, DW w) {
+invit_kernel(int n, DW w, unsigned salt) {
   extern __shared__ float zsh[];
   const int r = *w.rank;
   const int ncl = w.cls[0];
@@ -956,7 +957,7 @@ invit_kernel(int n, DW w) {
     LU[o] = __frcp_rn((fabsf(p0) < tiny) ? ((p0 < 0.f) ? -tiny : tiny) : p0);
     LU[pl + o] = 0.f;
     LU[2 * pl + o] = 0.f;
-    for (int a = 0; a < r; ++a) Z[a * zld + t] = start_value(a, jv);
+    for (int a = 0; a < r; ++a) Z[a * zld + t] = start_value(a, jv, salt);
   }
   for (int itr = 0; itr < kInvIters; ++itr) {
     for (int t = tid; t < m; t += kInvThreads) {
@@ -1778,7 +1779,7 @@ size_t dense_work_doubles(int n) {
 
 void dense_eig(const double* Ahat, const double* Mhat, int n, double sigma, int k, double* theta,
                double* Y, int* rank, double* work, double* quality, double drop_tol, int nq, cudaStream_t s,
-               int sel_first) {
+               int sel_first, int salt) {
   if (n < 1 || n > kMaxDense || k < 1 || k > n) fail(BMG_ERR_INVALID_ARG, "dense_eig: need 1 <= k <= n <= 224");
   TraceRange trace("enriched eigensolve");
   prof_begin(KC_DENSE, s);
@@ -1826,7 +1827,7 @@ void dense_eig(const double* Ahat, const double* Mhat, int n, double sigma, int 
   }
   const size_t ism = sizeof(float) * ((size_t)n * kInvSmemMembers + kInvLuFloats);
   BMG_CUDA(cudaFuncSetAttribute(invit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ism));
-  invit_kernel<<<n, kInvThreads, ism, s>>>(n, w);
+  invit_kernel<<<n, kInvThreads, ism, s>>>(n, w, (unsigned)salt);
   check_launch("invit_kernel");
   backtr_kernel<<<(n + 2 * kBackWarps - 1) / (2 * kBackWarps), kBackWarps * 32, 0, s>>>(n, w);
   check_launch("backtr_kernel");
