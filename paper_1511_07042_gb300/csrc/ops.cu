@@ -64,6 +64,176 @@ __device__ __forceinline__ void stv(float* p, size_t i, const float (&v)[4]) {
   reinterpret_cast<float4*>(p)[i] = make_float4(v[0], v[1], v[2], v[3]);
 }
 
+// ---- float64 rows in integer arithmetic ---------------------------------------
+// GB300 retires a float64 multiply-add per warp and scheduler every 64 cycles, an
+// integer add every one, a shift or logic operation every two and a 32 x 32 + 64
+// multiply-add in 2.4 (measured).  The row products of float64 blocks are therefore
+// formed in integers, except the first NF nonzeros, which keep the float64 unit busy
+// meanwhile and are added last:
+//   a = A' 2^(Ea - 1081), |A'| < 2^59, Ea the largest exponent field of the row's values;
+//   x = X' 2^(Ex - 1082), |X'| < 2^60, Ex the largest one among the row's values of X in
+//   that column; each split into signed 32-bit halves, A' = ah 2^32 + al;
+//   sum a x = (sum ah xh) 2^64 + (sum ah xl + al xh) 2^32, both sums exact in int64 over
+//   kFixNnz nonzeros, and one rounding to nearest at the end.
+// Dropped: al xl and the bits that the alignment shifts out, together below 2^-56 of
+// max|a| max|x| a term.  A float64 sum rounds each of its partial sums at 2^-53.  Against
+// exact sums of 7 products the integer sum's error is at most the float64 sum's (3e-17
+// against 7e-17 of sum |a x| in the mean over Laplacian rows, 5.6e-16 against 5.4e-16 at
+// most over rows of random exponents) where some product of the row comes within
+// kFixSlack bits of max|a| max|x|.  Rows without such a product (large x that all meet
+// small a), rows longer than kFixNnz, and values outside a band of exponents (zeros among
+// normal values excepted; Inf, NaN and subnormals fall outside) take the float64 loop.
+// Result and error do not depend on the lanes per row.
+// Measured, 655362 x 128: [AX | MX] 1924 -> 1194 us (NF = 2; 1418 and 1350 us with 1 and
+// 3); now bound by the issue of about 55 integer instructions per product pair.
+constexpr int kFixNnz = 7;     // a vertex of a subdivided surface and its six neighbours
+constexpr int kFixSlack = 3;
+struct FixEntry {
+  int ah, al, mh, ml;   // halves of A' and M'
+};
+struct FixIndex {
+  int col, slack;       // column; Ea - ea (low half) and Em - em (high half), at most 0x3fff
+};
+struct FixStage {       // one row of a warp
+  FixEntry e[8];
+  FixIndex j[8];
+};
+__device__ __forceinline__ int exp_field(double v) { return (__double2hiint(v) >> 20) & 0x7FF; }
+// v 2^(1081 - emax) (drop = 5) or v 2^(1082 - emax) (drop = 4), rounded towards zero, as
+// h 2^32 + l with a signed l; sh = emax - exponent field of v
+__device__ __forceinline__ void fix_halves(double v, int sh, int drop, int& h, int& l) {
+  const int hi = __double2hiint(v), lo = __double2loint(v);
+  unsigned long long m = ((unsigned long long)(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | (unsigned)(lo << 11);
+  asm("shr.u64 %0, %1, %2;" : "=l"(m) : "l"(m), "r"(sh + drop));   // a shift past 63 gives 0
+  const long long s = (long long)(hi >> 31);
+  const long long w = ((long long)m ^ s) - s;
+  l = (int)w;
+  h = (int)(w >> 32) - (l >> 31);
+}
+// (hi 2^64 + mid 2^32) 2^(e - 2163): the two sums as one integer in units of 2^-60 of
+// max|a| max|x| (below 2^63: seven products below 2^119, units of 2^59), rounded to nearest
+__device__ __forceinline__ double fix_value(long long hi, long long mid, int e) {
+  const long long v = (hi << 5) + (mid >> 27);
+  const double d = __ll2double_rn(v);
+  return v == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + ((e - 2104) << 20), __double2loint(d));
+}
+
+template <int LPR, int CPL, bool WITH_M, int NF>
+__device__ __forceinline__ void gather_row_fixed(const int* __restrict__ col, const double* __restrict__ va,
+                                                 const double* __restrict__ vm, const double* __restrict__ X, int b,
+                                                 int len, int nch, int sl, FixStage* st, double (&aa)[CPL][2],
+                                                 double (&mm)[CPL][2]) {
+  // the row's values as integers, by the first lanes of the row
+  constexpr int NQ = LPR >= 8 ? 1 : 8 / LPR;
+  const bool small = len <= kFixNnz && len > NF;
+  double av[NQ], mv[NQ];
+  int jv[NQ], ea = 0, em = 0;
+#pragma unroll
+  for (int t = 0; t < NQ; ++t) {
+    const int q = sl + t * LPR;
+    const bool in = small && q < len;
+    jv[t] = in ? __ldcs(col + b + q) : 0;
+    av[t] = in ? __ldcs(va + b + q) : 0.0;
+    mv[t] = (WITH_M && in) ? __ldcs(vm + b + q) : 0.0;
+    if (q >= NF) {
+      ea = max(ea, exp_field(av[t]));
+      em = max(em, exp_field(mv[t]));
+    }
+  }
+#pragma unroll
+  for (int o = 1; o < (LPR < 8 ? LPR : 8); o <<= 1) {
+    ea = max(ea, __shfl_xor_sync(0xffffffffu, ea, o));
+    if (WITH_M) em = max(em, __shfl_xor_sync(0xffffffffu, em, o));
+  }
+  const int j0 = __shfl_sync(0xffffffffu, jv[0], 0, LPR);
+  if (LPR > 8) {
+    ea = __shfl_sync(0xffffffffu, ea, 0, LPR);
+    if (WITH_M) em = __shfl_sync(0xffffffffu, em, 0, LPR);
+  }
+  __syncwarp();                       // the warp's previous rows are read
+#pragma unroll
+  for (int t = 0; t < NQ; ++t) {
+    const int q = sl + t * LPR;
+    if (q < 8) {
+      FixEntry f;
+      const int xa = exp_field(av[t]), xm = exp_field(mv[t]);
+      if (q < NF) {
+        f = {__double2hiint(av[t]), __double2loint(av[t]), __double2hiint(mv[t]), __double2loint(mv[t])};
+      } else {
+        fix_halves(av[t], ea - xa, 5, f.ah, f.al);
+        fix_halves(mv[t], em - xm, 5, f.mh, f.ml);
+        if (xa == 0) f.ah = f.al = 0;   // zero (all zero or subnormal rows take the other path)
+        if (xm == 0) f.mh = f.ml = 0;
+      }
+      st->e[q] = f;
+      // an absent nonzero reads the row's first column again, with the value 0
+      st->j[q] = {q < len ? jv[t] : j0, (xa ? ea - xa : 0x3fff) | ((xm ? em - xm : 0x3fff) << 16)};
+    }
+  }
+  __syncwarp();
+  const bool row_ok = small && ea >= 130 && ea <= 1900 && (!WITH_M || (em >= 130 && em <= 1900));
+#pragma unroll
+  for (int u = 0; u < CPL; ++u) {
+    const int c = sl + LPR * u;
+    if (c >= nch) continue;
+    double x[kFixNnz][2];
+#pragma unroll
+    for (int q = 0; q < kFixNnz; ++q) ldv_ro(X, (size_t)st->j[q].col * nch + c, x[q]);
+#pragma unroll
+    for (int z = 0; z < 2; ++z) {
+      int ex = 0;
+      unsigned best = 0xffffffffu;
+      long long ha = 0, ma = 0, hm = 0, lm = 0;
+#pragma unroll
+      for (int q = NF; q < kFixNnz; ++q) ex = max(ex, exp_field(x[q][z]));
+#pragma unroll
+      for (int q = NF; q < kFixNnz; ++q) {
+        const FixEntry f = st->e[q];
+        const int sh = ex - exp_field(x[q][z]);
+        int xh, xl;
+        fix_halves(x[q][z], sh, 4, xh, xl);
+        best = __vminu2(best, (unsigned)(st->j[q].slack + sh * 0x10001));
+        ha += (long long)f.ah * xh;
+        ma += (long long)f.ah * xl;
+        ma += (long long)f.al * xh;
+        if (WITH_M) {
+          hm += (long long)f.mh * xh;
+          lm += (long long)f.mh * xl;
+          lm += (long long)f.ml * xh;
+        }
+      }
+      const bool ok = row_ok && ex >= 130 && ex + ea >= 1200 && ex + ea <= 3000 && ex <= 1900 &&
+                      (best & 0xffffu) <= kFixSlack &&
+                      (!WITH_M || (ex + em >= 1200 && ex + em <= 3000 && (best >> 16) <= kFixSlack));
+      double s = 0.0, t = 0.0;
+      if (ok) {
+        s = fix_value(ha, ma, ea + ex);
+        if (WITH_M) t = fix_value(hm, lm, em + ex);
+      } else {
+        bool zero = row_ok && ex == 0;   // a padding column: nothing to add
+#pragma unroll
+        for (int q = NF; q < kFixNnz; ++q) zero = zero && x[q][z] == 0.0;
+        if (!zero)
+          for (int p = b + (small ? NF : 0); p < b + len; ++p) {
+            const double xv = __ldg(X + ((size_t)col[p] * nch + c) * 2 + z);
+            s = fma(va[p], xv, s);
+            if (WITH_M) t = fma(vm[p], xv, t);
+          }
+      }
+      if (small) {
+#pragma unroll
+        for (int q = 0; q < NF; ++q) {
+          const FixEntry f = st->e[q];
+          s = fma(__hiloint2double(f.ah, f.al), x[q][z], s);
+          if (WITH_M) t = fma(__hiloint2double(f.mh, f.ml), x[q][z], t);
+        }
+      }
+      aa[u][z] = s;
+      if (WITH_M) mm[u][z] = t;
+    }
+  }
+}
+
 // aa += A_row X, mm += M_row X for one CSR row owned by LPR lanes (pattern and values
 // streamed, neighbour rows of X gathered through the read-only path).  The row's
 // nonzeros are taken G at a time: lane q of the row's lanes loads nonzero q's column
@@ -72,42 +242,25 @@ __device__ __forceinline__ void stv(float* p, size_t i, const float (&v)[4]) {
 // in flight instead of one dependent load chain per nonzero.  The products are added
 // in the order of the nonzeros, as one nonzero at a time would.  Every lane of the
 // warp must call this (len = 0 for lanes without a row): the loop bound is the
-// warp's longest row.  (float32 blocks; float64 blocks take one nonzero at a time.)
+// warp's longest row.  float64 blocks: gather_row_fixed (st: the row's shared staging,
+// NF: nonzeros left to the float64 unit).
 template <typename T, int LPR, int CPL>
 struct GatherWidth {
   static constexpr int regs = CPL * Chunk<T>::W * (int)(sizeof(T) / 4);   // 32-bit registers per nonzero
   static constexpr int G0 = 32 / regs < 2 ? 2 : 32 / regs;
   static constexpr int G = G0 < LPR ? G0 : LPR;
 };
-template <typename T, int LPR, int CPL, bool WITH_M = true>
+template <typename T, int LPR, int CPL, bool WITH_M = true, int NF = 0>
 __device__ __forceinline__ void gather_row(const int* __restrict__ col, const T* __restrict__ va,
                                            const T* __restrict__ vm, const T* __restrict__ X, int b, int len,
-                                           int nch, int sl, T (&aa)[CPL][Chunk<T>::W],
+                                           int nch, int sl, FixStage* st, T (&aa)[CPL][Chunk<T>::W],
                                            T (&mm)[CPL][Chunk<T>::W]) {
   // WITH_M = false: only A x (mm untouched), for shifted problems with shift 0
   constexpr int W = Chunk<T>::W;
-  if (sizeof(T) == 8) {
-    // float64 blocks: the sweeps are bound by the FP64 pipe, not by memory latency,
-    // so one nonzero at a time (no shuffles competing for issue slots)
-    for (int p = b; p < b + len; ++p) {
-      const int j = __ldcs(col + p);
-      const T a = __ldcs(va + p), m = WITH_M ? __ldcs(vm + p) : T(0);
-#pragma unroll
-      for (int u = 0; u < CPL; ++u) {
-        const int c = sl + LPR * u;
-        if (c < nch) {
-          T x[W];
-          ldv_ro(X, (size_t)j * nch + c, x);
-#pragma unroll
-          for (int z = 0; z < W; ++z) {
-            aa[u][z] = fma(a, x[z], aa[u][z]);
-            if (WITH_M) mm[u][z] = fma(m, x[z], mm[u][z]);
-          }
-        }
-      }
-    }
+  if constexpr (sizeof(T) == 8) {
+    gather_row_fixed<LPR, CPL, WITH_M, NF>(col, va, vm, X, b, len, nch, sl, st, aa, mm);
     return;
-  }
+  } else {
   constexpr int G = GatherWidth<T, LPR, CPL>::G;
   const int maxlen = __reduce_max_sync(0xffffffffu, len);
   for (int p0 = 0; p0 < maxlen; p0 += G) {
@@ -151,14 +304,27 @@ __device__ __forceinline__ void gather_row(const int* __restrict__ col, const T*
       }
     }
   }
+  }
 }
 
-// 1/d for the smoother update.  FP64: an FP32 seed refined by two Newton-Raphson
-// steps y <- y (2 - d y) in FP64 (the relative error squares: 2^-23 -> 2^-46 -> below
-// rounding), a handful of FP64 operations instead of a full-precision division.  The
-// shifted diagonal d is far inside the FP32 range.  FP32: the correctly rounded
-// reciprocal.
+// 1/d for the smoother update.  FP64: an FP32 seed y (relative error below 2^-22) and one
+// step of third order, y (1 + e + e^2) with e = 1 - d y, leave the rounding of the last
+// operation.  The seed is read from and returned to the float64 bits by integer
+// operations: a conversion between the two costs as much as a float64 operation (64
+// cycles a warp).  Values outside 2^-100 .. 2^100 take the conversions and two Newton steps.
+// FP32: the correctly rounded reciprocal.
 __device__ __forceinline__ double recip(double d) {
+  const int hi = __double2hiint(d);
+  const unsigned ah = (unsigned)hi & 0x7fffffffu;
+  if (ah - 0x39b00000u < 0x46300000u - 0x39b00000u) {   // 2^-100 <= |d| < 2^100
+    const float f = __uint_as_float(((ah - 0x38000000u) << 3) | ((unsigned)__double2loint(d) >> 29));
+    float yf;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(yf) : "f"(f));
+    const unsigned yb = __float_as_uint(yf);
+    const double y = __hiloint2double((int)(((yb >> 3) + 0x38000000u) | ((unsigned)hi & 0x80000000u)), (int)(yb << 29));
+    const double e = fma(-d, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+  }
   double y = (double)__frcp_rn((float)d);
   y = y * fma(-d, y, 2.0);
   y = y * fma(-d, y, 2.0);
@@ -170,19 +336,24 @@ __device__ __forceinline__ float recip(float d) { return __frcp_rn(d); }
 // Row tiling: LPR lanes per row (32 / LPR rows per warp), CPL 16-byte chunks per lane
 // (chunks sl, sl + LPR, ...), blockDim.x / 32 warps per block; picked per level size
 // and block width by the autotuner (tune_rows).
+// float64: at most 8 warps a block and 80 registers, so that three blocks are resident
+// (24 warps hide the gathers' latency; 16 warps at 102 registers measured 1450 us at
+// 655362 x 128, all nonzeros in integers).
 // Row groups (a group: the rows of one pass of a CTA's warps) are dealt to the CTAs in
 // chunks of `groups` consecutive groups, round robin: an SM walks short contiguous
 // stretches of the Morton row order (neighbour rows of X found in its L1), while all
 // SMs together stay within a window of the order that L2 holds (neighbours shared
 // across chunks found in L2).
 template <typename T, int LPR, int CPL>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512, sizeof(T) == 8 ? 3 : 1)
 spmm_am_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
                const T* __restrict__ va, const T* __restrict__ vm,
                const T* __restrict__ X, int n, int nch, T* __restrict__ AX,
                T* __restrict__ MX, const int* __restrict__ order, int groups) {
   constexpr int W = Chunk<T>::W;
   constexpr int RPW = 32 / LPR;
+  __shared__ FixStage stage[sizeof(T) == 8 ? 8 * RPW : 1];   // float64 blocks: a row of each warp part
+  FixStage* st = stage + (sizeof(T) == 8 ? (threadIdx.x >> 5) * RPW + (threadIdx.x & 31) / LPR : 0);
   const int lane = threadIdx.x & 31, sl = lane % LPR;
   const int per_group = (blockDim.x >> 5) * RPW;
   const int ngroups = (n + per_group - 1) / per_group;
@@ -198,7 +369,7 @@ spmm_am_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
 #pragma unroll
       for (int q = 0; q < W; ++q) { aa[u][q] = T(0); mm[u][q] = T(0); }
     const int b = live ? row_ptr[row] : 0;
-    gather_row<T, LPR, CPL>(col, va, vm, X, b, live ? row_ptr[row + 1] - b : 0, nch, sl, aa, mm);
+    gather_row<T, LPR, CPL, true, 2>(col, va, vm, X, b, live ? row_ptr[row + 1] - b : 0, nch, sl, st, aa, mm);
     if (!live) continue;
 #pragma unroll
     for (int u = 0; u < CPL; ++u) {
@@ -219,7 +390,7 @@ spmm_am_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
 // ZS: every shift is zero (the shifted problems of a solve at sigma = 0): r = b - A x
 // and d = dA_i, so M and its diagonal are not read and 1/d is formed once per row.
 template <typename T, int LPR, int CPL, int MODE, bool ZS>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512, sizeof(T) == 8 ? 3 : 1)
 row_update_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
                   const T* __restrict__ va, const T* __restrict__ vm,
                   const T* __restrict__ da, const T* __restrict__ dm,
@@ -228,6 +399,8 @@ row_update_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
                   int nch, T omega, int groups) {
   constexpr int W = Chunk<T>::W;
   constexpr int RPW = 32 / LPR;
+  __shared__ FixStage stage[sizeof(T) == 8 ? 8 * RPW : 1];   // float64 blocks: a row of each warp part
+  FixStage* st = stage + (sizeof(T) == 8 ? (threadIdx.x >> 5) * RPW + (threadIdx.x & 31) / LPR : 0);
   const int lane = threadIdx.x & 31, sl = lane % LPR;
   const int per_group = (blockDim.x >> 5) * RPW;
   const int ngroups = (nrows + per_group - 1) / per_group;
@@ -243,7 +416,7 @@ row_update_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
 #pragma unroll
       for (int q = 0; q < W; ++q) { aa[u][q] = T(0); mm[u][q] = T(0); }
     const int b = live ? row_ptr[row] : 0;
-    gather_row<T, LPR, CPL, !ZS>(col, va, vm, X, b, live ? row_ptr[row + 1] - b : 0, nch, sl, aa, mm);
+    gather_row<T, LPR, CPL, !ZS, ZS ? 2 : 0>(col, va, vm, X, b, live ? row_ptr[row + 1] - b : 0, nch, sl, st, aa, mm);
     if (!live) continue;
     const T dai = da[row], dmi = ZS ? T(0) : dm[row];
     const T rd0 = (ZS && MODE != 2) ? recip(dai) : T(0);
@@ -290,13 +463,15 @@ row_update_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
 // of one colour of a distance-2 colouring share no column, so the updates of a launch
 // touch disjoint rows of X and no row they read is written by another row.
 template <typename T, int LPR, int CPL>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(256)
 kaczmarz_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col, const T* __restrict__ va,
                 const T* __restrict__ vm, const T* __restrict__ na, const T* __restrict__ nam,
                 const T* __restrict__ nm, const int* __restrict__ rows, int nrows, T* X,
                 const T* __restrict__ B, const T* __restrict__ shift, int nch, T omega) {
   constexpr int W = Chunk<T>::W;
   constexpr int RPW = 32 / LPR;
+  __shared__ FixStage stage[sizeof(T) == 8 ? 8 * RPW : 1];   // float64 blocks: a row of each warp part
+  FixStage* st = stage + (sizeof(T) == 8 ? (threadIdx.x >> 5) * RPW + (threadIdx.x & 31) / LPR : 0);
   const int lane = threadIdx.x & 31, sl = lane % LPR;
   const int w = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * RPW + lane / LPR;
   const bool live = w < nrows;
@@ -308,7 +483,7 @@ kaczmarz_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col, co
     for (int q = 0; q < W; ++q) { aa[u][q] = T(0); mm[u][q] = T(0); }
   const int b = live ? row_ptr[row] : 0;
   const int e = live ? row_ptr[row + 1] : 0;
-  gather_row<T, LPR, CPL>(col, va, vm, X, b, e - b, nch, sl, aa, mm);
+  gather_row<T, LPR, CPL>(col, va, vm, X, b, e - b, nch, sl, st, aa, mm);
   if (!live) return;
   const T n_a = na[row], n_am = nam[row], n_m = nm[row];
   T coef[CPL][W], sv[CPL][W];
@@ -831,6 +1006,7 @@ RowCfg tune_rows(int kind, int tsize, int nch, int n, cudaStream_t s, F&& launch
   for (int sh = 0; sh < kNumShapes; ++sh) {
     if (!shape_ok(sh, nch)) continue;
     for (int wpb : kWPB) {
+      if (tsize == 8 && wpb > 8) continue;   // float64 row kernels: 256 threads at most
       RowCfg c;
       c.shape = sh;
       c.wpb = wpb;
