@@ -17,6 +17,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <thread>
 #include <vector>
@@ -43,6 +44,94 @@ void check_launch(const char* what) {
   count_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) fail(BMG_ERR_CUDA, std::string("launch of ") + what + ": " + cudaGetErrorString(e));
+}
+
+// ------------------------------------------------------ workspace pool ----
+namespace {
+struct PoolItem {
+  void* ptr;
+  size_t bytes;
+  int* flag;
+  int dev;
+};
+std::mutex g_pool_mu;
+std::vector<PoolItem> g_pool;   // idle buffers
+
+void pool_free(const PoolItem& it) {
+  int cur = 0;
+  cudaGetDevice(&cur);
+  if (cur != it.dev) cudaSetDevice(it.dev);
+  cudaFree(it.ptr);
+  cudaFreeHost(it.flag);
+  if (cur != it.dev) cudaSetDevice(cur);
+}
+}  // namespace
+
+void pool_trim() {
+  std::vector<PoolItem> all;
+  {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    all.swap(g_pool);
+  }
+  for (const PoolItem& it : all) pool_free(it);
+}
+
+Workspace::Workspace(size_t bytes, cudaStream_t s) : s_(s) {
+  check_cuda(cudaGetDevice(&dev_), "cudaGetDevice");
+  {
+    // the smallest idle buffer that is large enough
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    size_t best = g_pool.size();
+    for (size_t q = 0; q < g_pool.size(); ++q)
+      if (g_pool[q].dev == dev_ && g_pool[q].bytes >= bytes &&
+          (best == g_pool.size() || g_pool[q].bytes < g_pool[best].bytes))
+        best = q;
+    if (best < g_pool.size()) {
+      ptr_ = g_pool[best].ptr;
+      bytes_ = g_pool[best].bytes;
+      flag_ = g_pool[best].flag;
+      g_pool.erase(g_pool.begin() + best);
+    }
+  }
+  if (!ptr_) {
+    bytes_ = (bytes + 0xFFFFF) & ~(size_t)0xFFFFF;   // whole megabytes, so that calls of near sizes share
+    cudaError_t e = cudaMalloc(&ptr_, bytes_);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      pool_trim();
+      e = cudaMalloc(&ptr_, bytes_);
+    }
+    if (e == cudaSuccess) {
+      e = cudaHostAlloc(&flag_, sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped);
+      if (e != cudaSuccess) cudaFree(ptr_);
+    }
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      ptr_ = nullptr;
+      fail(BMG_ERR_OOM, "workspace of " + std::to_string(bytes_) + " bytes: " + cudaGetErrorString(e));
+    }
+  }
+  *flag_ = 0;
+}
+
+Workspace::~Workspace() {
+  if (!ptr_) return;
+  if (!idle_) cudaStreamSynchronize(s_);
+  std::vector<PoolItem> drop;
+  {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    g_pool.push_back({ptr_, bytes_, flag_, dev_});
+    // over the limit: the oldest idle buffers of the device go
+    size_t held = 0;
+    for (const PoolItem& it : g_pool) held += it.dev == dev_ ? it.bytes : 0;
+    for (size_t q = 0; q < g_pool.size() && held > kPoolBytes;) {
+      if (g_pool[q].dev != dev_) { ++q; continue; }
+      held -= g_pool[q].bytes;
+      drop.push_back(g_pool[q]);
+      g_pool.erase(g_pool.begin() + q);
+    }
+  }
+  for (const PoolItem& it : drop) pool_free(it);
 }
 
 namespace {
@@ -128,6 +217,7 @@ extern "C" const char* bmg_last_error(void) { return g_last_error.c_str(); }
 extern "C" void bmg_destroy(bmg_problem* p) {
   if (!p) return;
   try { delete p; } catch (...) {}
+  pool_trim();
 }
 
 extern "C" bmg_status bmg_assemble(const double* verts, int n_verts, const int* tris, int n_tris,
@@ -406,18 +496,19 @@ extern "C" bmg_status bmg_gram(const double* X, const double* Y, int n, int k, i
     if (!X || !Y || !G || n < 1 || k < 1 || k > 160 || ld < k || ld > kGramMaxLd)
       fail(BMG_ERR_INVALID_ARG, "bad gram arguments (1 <= k <= 160, k <= ld <= 800)");
     const int parts = gram_parts(n);
-    DBuf<double> partial((size_t)parts * k * k);
-    gram(X, Y, n, k, ld, G, partial.get(), parts, (cudaStream_t)stream);
+    Workspace ws(sizeof(double) * (size_t)parts * k * k, (cudaStream_t)stream);
+    gram(X, Y, n, k, ld, G, ws.get<double>(), parts, (cudaStream_t)stream);
     BMG_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
+    ws.idle();
   });
 }
 
-// Reads a device error flag raised by a tensor-core kernel after the stream is idle.
-static void check_tc_flag(const int* flag, cudaStream_t s) {
-  int h = 0;
-  BMG_CUDA(cudaMemcpyAsync(&h, flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+// Waits for a call's work and reads the flag that a tensor-core kernel raises when a wait
+// expires.
+static void finish_tc(Workspace& ws, cudaStream_t s) {
   BMG_CUDA(cudaStreamSynchronize(s));
-  if (h) fail(BMG_ERR_TIMEOUT, "a bounded wait in a tensor-core kernel expired");
+  ws.idle();
+  if (*static_cast<volatile int*>(ws.flag())) fail(BMG_ERR_TIMEOUT, "a bounded wait in a tensor-core kernel expired");
 }
 
 template <typename T>
@@ -426,11 +517,9 @@ static void gram_tc_entry(const T* X, const T* Y, int n, int k, int ld, double* 
     fail(BMG_ERR_INVALID_ARG, "bad gram arguments (1 <= k <= 128, ld >= k)");
   cudaStream_t s = (cudaStream_t)stream;
   const int parts = gram_tc_parts(n, k);
-  DBuf<double> partial((size_t)parts * k * k);
-  DBuf<int> flag(1);
-  BMG_CUDA(cudaMemsetAsync(flag.get(), 0, sizeof(int), s));
-  gram_tc(X, Y, n, k, ld, G, partial.get(), parts, flag.get(), s, false);
-  check_tc_flag(flag.get(), s);
+  Workspace ws(sizeof(double) * (size_t)parts * k * k, s);
+  gram_tc(X, Y, n, k, ld, G, ws.get<double>(), parts, ws.flag(), s, false);
+  finish_tc(ws, s);
 }
 
 extern "C" bmg_status bmg_gram_tc(const double* X, const double* Y, int n, int k, int ld, double* G, void* stream) {
@@ -451,12 +540,11 @@ extern "C" bmg_status bmg_gram_tc_f32(const float* X, const float* Y, int n, int
 extern "C" bmg_status bmg_tc_timeout_selftest(void* stream) {
   return guarded([&] {
     cudaStream_t s = (cudaStream_t)stream;
-    DBuf<double> X((size_t)4096 * 64), G((size_t)64 * 64), partial((size_t)gram_tc_parts(4096, 64) * 64 * 64);
-    DBuf<int> flag(1);
+    DBuf<double> X((size_t)4096 * 64), G((size_t)64 * 64);
+    Workspace ws(sizeof(double) * (size_t)gram_tc_parts(4096, 64) * 64 * 64, s);
     BMG_CUDA(cudaMemsetAsync(X.get(), 0, sizeof(double) * 4096 * 64, s));
-    BMG_CUDA(cudaMemsetAsync(flag.get(), 0, sizeof(int), s));
-    gram_tc_timeout_selftest(X.get(), G.get(), partial.get(), flag.get(), s);
-    check_tc_flag(flag.get(), s);
+    gram_tc_timeout_selftest(X.get(), G.get(), ws.get<double>(), ws.flag(), s);
+    finish_tc(ws, s);
     fail(BMG_ERR_CUDA, "tc timeout self-test: the bounded waits did not expire");
   });
 }
@@ -471,11 +559,9 @@ static void expand_entry(const T* Z, const T* X, const double* Yx, int n, int k,
   cudaStream_t s = (cudaStream_t)stream;
   if (tensor_cores) {
     if (k > kTcMaxK) fail(BMG_ERR_INVALID_ARG, "tensor-core expand: k <= 128");
-    DBuf<unsigned char> scratch(expand_tc_scratch_bytes(k));
-    DBuf<int> flag(1);
-    BMG_CUDA(cudaMemsetAsync(flag.get(), 0, sizeof(int), s));
-    expand_tc(Z, X, Yx, n, k, ld, ldy, U, scratch.get(), flag.get(), s);
-    check_tc_flag(flag.get(), s);
+    Workspace ws(expand_tc_scratch_bytes(k), s);
+    expand_tc(Z, X, Yx, n, k, ld, ldy, U, ws.get<unsigned char>(), ws.flag(), s);
+    finish_tc(ws, s);
   } else {
     expand<T>(Z, X, Yx, n, k, ld, ldy, U, s);
     BMG_CUDA(cudaStreamSynchronize(s));
@@ -497,11 +583,13 @@ extern "C" bmg_status bmg_dense_eig(const double* Ahat, const double* Mhat, int 
   return guarded([&] {
     if (!Ahat || !Mhat || !theta || !Y) fail(BMG_ERR_INVALID_ARG, "null pointer");
     if (n < 1 || n > 224 || k < 1 || k > n) fail(BMG_ERR_INVALID_ARG, "need 1 <= k <= n <= 224");
-    DBuf<double> work(dense_work_doubles(n));
-    DBuf<int> rk(1);
-    dense_eig(Ahat, Mhat, n, sigma, k, theta, Y, rank_out ? rank_out : rk.get(), work.get(), nullptr,
-              kDropFP64, 0, (cudaStream_t)stream);
+    const size_t wn = dense_work_doubles(n);
+    Workspace ws(sizeof(double) * (wn + 1), (cudaStream_t)stream);
+    int* rk = reinterpret_cast<int*>(ws.get<double>() + wn);
+    dense_eig(Ahat, Mhat, n, sigma, k, theta, Y, rank_out ? rank_out : rk, ws.get<double>(), nullptr, kDropFP64, 0,
+              (cudaStream_t)stream);
     BMG_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
+    ws.idle();
   });
 }
 
@@ -1493,9 +1581,10 @@ extern "C" bmg_status bmg_gram_f32(const float* X, const float* Y, int n, int k,
     if (!X || !Y || !G || n < 1 || k < 1 || k > 160 || ld < k || (ld & 3) || ld > kGramMaxLd)
       fail(BMG_ERR_INVALID_ARG, "bad gram arguments (1 <= k <= 160, k <= ld <= 800, ld % 4 == 0)");
     const int parts = gram_parts(n);
-    DBuf<double> partial((size_t)parts * k * k);
-    gram(X, Y, n, k, ld, G, partial.get(), parts, (cudaStream_t)stream);
+    Workspace ws(sizeof(double) * (size_t)parts * k * k, (cudaStream_t)stream);
+    gram(X, Y, n, k, ld, G, ws.get<double>(), parts, (cudaStream_t)stream);
     BMG_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
+    ws.idle();
   });
 }
 

@@ -63,11 +63,17 @@ struct DBuf {
   T* get() const { return ptr; }
 };
 
+void pool_trim();
 template <typename T>
 void DBuf<T>::alloc(size_t count) {
   release();
   if (count == 0) return;
   cudaError_t e = cudaMalloc(&ptr, count * sizeof(T));
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    pool_trim();
+    e = cudaMalloc(&ptr, count * sizeof(T));
+  }
   if (e != cudaSuccess) {
     ptr = nullptr;
     cudaGetLastError();
@@ -76,6 +82,35 @@ void DBuf<T>::alloc(size_t count) {
   }
   n = count;
 }
+
+// Workspace of one synchronous call (partial sums, digits, the dense eigensolve's scratch),
+// taken from a process-wide pool so that a call neither allocates nor frees device memory
+// (a cudaMalloc and cudaFree of more than 2 MB take about 130 us, as long as the kernels of
+// a small call).  A buffer serves one call at a time on any stream: the destructor waits
+// for the stream unless idle() was called after a synchronisation.  The pool keeps at most
+// kPoolBytes per device, is emptied by every bmg_destroy and when a device allocation
+// fails, and takes calls from several threads.  flag() is a pinned host word that the
+// call's kernels may raise; it is zero on construction.
+class Workspace {
+ public:
+  Workspace(size_t bytes, cudaStream_t s);
+  ~Workspace();
+  Workspace(const Workspace&) = delete;
+  Workspace& operator=(const Workspace&) = delete;
+  template <typename T> T* get() const { return static_cast<T*>(ptr_); }
+  int* flag() const { return flag_; }
+  void idle() { idle_ = true; }
+
+ private:
+  void* ptr_ = nullptr;
+  size_t bytes_ = 0;
+  int* flag_ = nullptr;
+  int dev_ = 0;
+  cudaStream_t s_;
+  bool idle_ = false;
+};
+constexpr size_t kPoolBytes = 64u << 20;
+void pool_trim();   // frees the pool's buffers that no call holds
 
 // ----------------------------------------------------------- structures ----
 // One refinement of the surface mesh (refinement 0 = the input mesh).
