@@ -744,21 +744,35 @@ gram_f32_kernel(const float* __restrict__ X, const float* __restrict__ Y, int n,
       if (ti + a < k && tj + b < k) out[(ti + a) * k + tj + b] = (double)s[a][b] + (double)c[a][b];
 }
 
-// G[q] = sum of the block partials in block order.  With sym (a k x k Gram of which
-// only the tiles on and above the diagonal were formed) an entry below the diagonal
-// tiles takes its mirror.
-__global__ void gram_reduce_kernel(const double* __restrict__ partial, int nparts, int kk,
-                                   double* __restrict__ G, int k = 0, int sym = 0) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= kk) return;
-  int src = q;
-  if (sym) {
-    const int i = q / k, j = q % k;
-    if (i / 4 > j / 4) src = j * k + i;
-  }
+// G[q] = sum of the block partials: kRedSlices threads an output take every kRedSlices-th
+// partial in order, and their sums are added in order (the partials of one output are a
+// stride apart, so one thread an output waits for one load after another: 15 us for 76
+// partials of 128 x 128).  With sym (a k x k Gram of which only the tiles on and above the
+// diagonal were formed) an entry below the diagonal tiles takes its mirror.
+constexpr int kRedSlices = 8, kRedOut = 32;
+__global__ void __launch_bounds__(kRedSlices * kRedOut)
+gram_reduce_kernel(const double* __restrict__ partial, int nparts, int kk, double* __restrict__ G, int k = 0,
+                   int sym = 0) {
+  __shared__ double sums[kRedSlices][kRedOut];
+  const int o = threadIdx.x % kRedOut, sl = threadIdx.x / kRedOut;
+  const int q = blockIdx.x * kRedOut + o;
   double s = 0.0;
-  for (int b = 0; b < nparts; ++b) s += partial[(size_t)b * kk + src];
-  G[q] = s;
+  if (q < kk) {
+    int src = q;
+    if (sym) {
+      const int i = q / k, j = q % k;
+      if (i / 4 > j / 4) src = j * k + i;
+    }
+#pragma unroll 4
+    for (int b = sl; b < nparts; b += kRedSlices) s += partial[(size_t)b * kk + src];
+  }
+  sums[sl][o] = s;
+  __syncthreads();
+  if (sl == 0 && q < kk) {
+#pragma unroll
+    for (int t = 1; t < kRedSlices; ++t) s += sums[t][o];
+    G[q] = s;
+  }
 }
 
 // ---- per-vector residual norms ----------------------------------------------
@@ -1215,7 +1229,7 @@ void gram(const double* X, const double* Y, int n, int k, int ld, double* G, dou
   else if (ntiles <= 8 * kGramThreads) gram_kernel<8><<<nparts, kGramThreads, smem, s>>>(X, Y, n, k, ld, rows_per_part, partial, sym ? 1 : 0);
   else fail(BMG_ERR_INVALID_ARG, "gram: k too large (k <= 180)");
   check_launch("gram_kernel");
-  gram_reduce_kernel<<<blocks_for(k * k, 256), 256, 0, s>>>(partial, nparts, k * k, G, k, sym ? 1 : 0);
+  gram_reduce_kernel<<<blocks_for(k * k, kRedOut), kRedSlices * kRedOut, 0, s>>>(partial, nparts, k * k, G, k, sym ? 1 : 0);
   check_launch("gram_reduce_kernel");
   prof_end(KC_GRAM, s, 16.0 * n * ld + 16.0 * nparts * k * k + 8.0 * k * k,
            (sym ? 1.0 : 2.0) * n * k * k + (sym ? 4.0 * n * k : 0.0));
@@ -1235,13 +1249,13 @@ void gram(const float* X, const float* Y, int n, int k, int ld, double* G, doubl
   const dim3 grid(nparts, (ntiles + kGram32Threads - 1) / kGram32Threads);
   gram_f32_kernel<<<grid, kGram32Threads, smem, s>>>(X, Y, n, k, ld, rows_per_part, partial, sym ? 1 : 0);
   check_launch("gram_f32_kernel");
-  gram_reduce_kernel<<<blocks_for(k * k, 256), 256, 0, s>>>(partial, nparts, k * k, G, k, sym ? 1 : 0);
+  gram_reduce_kernel<<<blocks_for(k * k, kRedOut), kRedSlices * kRedOut, 0, s>>>(partial, nparts, k * k, G, k, sym ? 1 : 0);
   check_launch("gram_reduce_kernel");
   prof_end(KC_GRAM, s, 8.0 * n * ld + 16.0 * nparts * k * k + 8.0 * k * k, 2.0 * n * k * k);
 }
 
 void gram_reduce(const double* partial, int nparts, int k, double* G, bool sym, cudaStream_t s) {
-  gram_reduce_kernel<<<blocks_for(k * k, 256), 256, 0, s>>>(partial, nparts, k * k, G, k, sym ? 1 : 0);
+  gram_reduce_kernel<<<blocks_for(k * k, kRedOut), kRedSlices * kRedOut, 0, s>>>(partial, nparts, k * k, G, k, sym ? 1 : 0);
   check_launch("gram_reduce_kernel");
 }
 
@@ -1254,7 +1268,7 @@ void eig_residuals(const T* AU, const T* MU, const T* U, const double* lam, int 
   eigres_kernel<T><<<nparts, threads, 2 * threads * sizeof(double), s>>>(AU, MU, U, lam, n, k, ld,
                                                                          rows_per_part, partial);
   check_launch("eigres_kernel");
-  gram_reduce_kernel<<<blocks_for(2 * k, 256), 256, 0, s>>>(partial, nparts, 2 * k, out);
+  gram_reduce_kernel<<<blocks_for(2 * k, kRedOut), kRedSlices * kRedOut, 0, s>>>(partial, nparts, 2 * k, out);
   check_launch("gram_reduce_kernel");
   prof_end(KC_SMALL, s, 3.0 * tb<T>() * n * ld, 5.0 * n * k);
 }
