@@ -8,10 +8,10 @@
 //   1. basis          the b_h-orthogonalisation of Alg. 2 step 3: Mhat scaled to unit
 //      diagonal and factored by Cholesky with diagonal pivoting; pivots below the drop
 //      tolerance mark basis vectors already in the span of the others, which are
-//      dropped (rank r).  basis_kernel [1 CTA] factors the whole of Mhat; the block
-//      form (qfactor_kernel, xsolve_kernel, schur_kernel, xfactor_cl_kernel) keeps the
-//      factor of a repeating leading block and factors the Schur complement of the
-//      new columns.
+//      dropped (rank r).  The block form (qfactor_kernel, xsolve_kernel, schur_kernel,
+//      xfactor_cl_kernel) keeps the factor of a repeating leading block and factors the
+//      Schur complement of the new columns; without such a block the whole of Mhat is the
+//      new block (a one-CTA factorisation took 698 us at n = 170, this one 390 us).
 //   2. trsm_kernel     [multi-CTA, FP64]  reduced standard matrix
 //      T = L^{-1} D P^T (Ahat - sigma Mhat) P D L^{-T}: two forward substitutions, one
 //      warp per column, L staged in shared memory.
@@ -31,6 +31,7 @@
 //   5. select / backsub  the k smallest |theta|; Y = D P L^{-T} W_sel.
 #include <algorithm>
 #include <cmath>
+#include <utility>
 
 #include <cooperative_groups.h>
 
@@ -45,7 +46,6 @@ constexpr int kMaxN = 320;
 constexpr int kMaxDense = 224;           // the FP32 stage keeps T (n^2 floats) in shared memory
 constexpr int kBig = 1024;               // threads of the single-CTA kernels
 constexpr int kFactorWarps = 32;         // warps of the pivoted Cholesky kernels (block form)
-constexpr int kBasisWarps = 32;          // warps of the whole-matrix pivoted Cholesky
 constexpr int kMaxCluster = 40;          // larger clusters keep the orthonormalising step only
 constexpr int kTile = 8;                 // output tile of the refinement products
 
@@ -217,50 +217,6 @@ __device__ int pchol(double* S, int n, int ld, double drop_tol, int* perm, doubl
   return rank;
 }
 
-// The whole of M-hat: unit-diagonal scaling, pivoted Cholesky, factor written as L
-// (row i holds L[i][0..i], pivot order) and Lt (row q holds column q of L).
-template <int NW>
-__global__ void __launch_bounds__(NW * 32, 1)
-basis_kernel(const double* __restrict__ Mhat, int n, DW w, int smemS, double drop_tol) {
-  extern __shared__ double dsm[];
-  double* S = smemS ? dsm : w.S;
-  __shared__ unsigned long long wk[32];
-  __shared__ int wi[32];
-  __shared__ int perm[kMaxN];
-  __shared__ double d[kMaxN], lcol[kMaxN], rls[kMaxN];
-  __shared__ int s_go;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  constexpr int nwarps = NW, NT = NW * 32;
-  for (int i = tid; i < n; i += NT) {
-    const double mii = Mhat[i * n + i];
-    d[i] = (mii > 0.0) ? 1.0 / sqrt(mii) : 0.0;
-    perm[i] = i;
-  }
-  __syncthreads();
-  for (int i = wid; i < n; i += nwarps)
-    for (int j = lane; j < n; j += 32) S[i * n + j] = 0.5 * (Mhat[i * n + j] + Mhat[j * n + i]) * (d[i] * d[j]);
-  __syncthreads();
-  const int rank = pchol<NW>(S, n, n, drop_tol, perm, lcol, rls, wk, wi, &s_go);
-  // write the factor: L (lower, rows in pivot order) and Lt, zero outside the first
-  // rank columns and above the diagonal
-  for (int i = wid; i < n; i += nwarps)
-    for (int q = lane; q < n; q += 32) {
-      const double v = (q <= i && q < rank) ? S[i * n + q] : 0.0;
-      w.L[i * n + q] = v;
-    }
-  for (int q = wid; q < n; q += nwarps)
-    for (int i = lane; i < n; i += 32) {
-      const double v = (q <= i && q < rank) ? S[i * n + q] : 0.0;
-      w.Lt[q * n + i] = v;
-    }
-  for (int i = tid; i < n; i += NT) {
-    w.perm[i] = perm[i];
-    w.d[i] = d[i];
-    if (i < rank) w.rl[i] = rls[i];
-  }
-  if (tid == 0) *w.rank = rank;
-}
-
 // --- Block form for M-hat = [[M_Q, C], [C^T, G]] whose leading nq x nq block M_Q (the
 // coarse space's own mass matrix) repeats from call to call: its factor is kept in the
 // workspace and recomputed only when the block changes; the block's new columns are
@@ -313,6 +269,74 @@ qfactor_kernel(const double* __restrict__ Mhat, int n, int nq, DW w, double drop
   if (tid == 0) { w.qflag[0] = (rank == nq) ? 1 : 2; w.qflag[1] = nq; }
 }
 
+// Unscaled forward substitution of one column by a warp: zs[i] = value of row i when it is
+// reached, then Ls[i][q] times it subtracted from the rows q > i (Ls: packed columns of an
+// r-row factor; lane l keeps rows l, l + 32, ... in acc).  A float64 instruction holds the
+// scheduler's float64 unit for 64 cycles, so the slot that holds the next row is updated
+// first and its value broadcast while the other slots' updates issue.  Slots are unrolled
+// (no selection by the row index), those that are finished skipped.
+template <int NS>
+__device__ __forceinline__ void forward_solve(const double* Ls, int r, int lane, double (&acc)[NS], double* zs) {
+  double a = __shfl_sync(0xffffffffu, acc[0], 0);
+#pragma unroll
+  for (int ti = 0; ti < NS; ++ti) {
+    for (int i = 32 * ti; i < min(r, 32 * ti + 32); ++i) {
+      if (lane == 0) zs[i] = a;
+      const int o = col_off(i, r) - i - 1;   // Ls[o + q] for q > i
+      double l[NS];
+#pragma unroll
+      for (int t = ti; t < NS; ++t) {
+        const int q = lane + 32 * t;
+        l[t] = (q > i && q < r) ? Ls[o + q] : 0.0;
+      }
+      const double ai = a;
+      acc[ti] = fma(-l[ti], ai, acc[ti]);
+      if ((i & 31) != 31) {
+        a = __shfl_sync(0xffffffffu, acc[ti], (i + 1) & 31);
+      } else if (ti + 1 < NS) {
+        acc[ti + 1 < NS ? ti + 1 : ti] = fma(-l[ti + 1 < NS ? ti + 1 : ti], ai, acc[ti + 1 < NS ? ti + 1 : ti]);
+        a = __shfl_sync(0xffffffffu, acc[ti + 1 < NS ? ti + 1 : ti], 0);
+      }
+#pragma unroll
+      for (int t = ti + 1; t < NS; ++t)
+        if (t > ti + 1 || (i & 31) != 31) acc[t] = fma(-l[t], ai, acc[t]);
+    }
+  }
+}
+// The same from the last row up: Lr[i][q] (packed rows, q < i) times row i's value
+// subtracted from the rows q < i.
+template <int NS>
+__device__ __forceinline__ void backward_solve(const double* Lr, int r, int lane, double (&acc)[NS], double* zs) {
+  double a = 0.0;
+#pragma unroll
+  for (int ti = NS - 1; ti >= 0; --ti) {
+    const int last = min(r, 32 * ti + 32) - 1;
+    if (last < 32 * ti) continue;
+    if (last == r - 1) a = __shfl_sync(0xffffffffu, acc[ti], last & 31);
+    for (int i = last; i >= 32 * ti; --i) {
+      if (lane == 0) zs[i] = a;
+      const double* li = Lr + i * (i - 1) / 2;        // li[q] for q < i
+      double l[NS];
+#pragma unroll
+      for (int t = 0; t <= ti; ++t) {
+        const int q = lane + 32 * t;
+        l[t] = (q < i) ? li[q] : 0.0;
+      }
+      const double ai = a;
+      acc[ti] = fma(-l[ti], ai, acc[ti]);
+      if ((i & 31) != 0) {
+        a = __shfl_sync(0xffffffffu, acc[ti], (i - 1) & 31);
+      } else if (ti > 0) {
+        acc[ti > 0 ? ti - 1 : 0] = fma(-l[ti > 0 ? ti - 1 : 0], ai, acc[ti > 0 ? ti - 1 : 0]);
+        a = __shfl_sync(0xffffffffu, acc[ti > 0 ? ti - 1 : 0], 31);
+      }
+#pragma unroll
+      for (int t = 0; t < ti; ++t)
+        if (t < ti - 1 || (i & 31) != 0) acc[t] = fma(-l[t], ai, acc[t]);
+    }
+  }
+}
+
 // W = L_Q^{-1} P_Q^T D_Q C D_X, one warp per new column x (as in trsm_kernel, L_Q
 // staged in shared memory, pre-scaled), output W[q][x] (row stride kx) in w.Z, and the
 // scaling d_X = 1 / sqrt(G_xx) into w.d[nq + x].
@@ -345,26 +369,17 @@ xsolve_kernel(const double* __restrict__ Mhat, int n, int nq, int kx, DW w) {
     }
     acc[t] = v;
   }
-  for (int i = 0; i < nq; ++i) {
-    const int ti = i >> 5;
-    double a = acc[0];
-#pragma unroll
-    for (int t = 1; t < NS; ++t)
-      if (ti == t) a = acc[t];
-    a = __shfl_sync(0xffffffffu, a, i & 31);
-    if (lane == 0) zs[i] = a;
-    const int o = col_off(i, nq) - i - 1;
-#pragma unroll
-    for (int t = 0; t < NS; ++t) {
-      if (t >= ti) {
-        const int q = lane + 32 * t;
-        const double l = (q > i && q < nq) ? Ls[o + q] : 0.0;
-        acc[t] = fma(-l, a, acc[t]);
-      }
-    }
-  }
+  forward_solve<NS>(Ls, nq, lane, acc, zs);
   __syncwarp();
   for (int q = lane; q < nq; q += 32) w.Z[q * kx + x] = zs[q] * w.qrl[q];
+}
+
+// Unit-diagonal scaling of the whole of M-hat (nq = 0), as xsolve_kernel's for the new columns.
+__global__ void scaling_kernel(const double* __restrict__ Mhat, int n, DW w) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double mii = Mhat[(size_t)i * n + i];
+  w.d[i] = (mii > 0.0) ? 1.0 / sqrt(mii) : 0.0;
 }
 
 // S_X = D_X sym(G) D_X - W^T W (kx x kx, row stride kx) into w.S; 8 x 8 output tiles on
@@ -383,7 +398,8 @@ schur_kernel(const double* __restrict__ Mhat, int n, int nq, int kx, DW w) {
 }
 
 // Pivoted Cholesky of S_X and assembly of the factor of the whole of M-hat in the
-// layout basis_kernel writes (L, Lt, rl, perm, d, rank).  A deficient M_Q gives rank 0.
+// layout of the solves below (L: row i holds L[i][0..i] in pivot order; Lt: row q holds
+// column q of L; rl, perm, d, rank).  A deficient M_Q gives rank 0.
 // The factorisation runs on a cluster of kXC CTAs, one per SM: the update, the bulk of
 // the FP64 work, then runs on kXC SMs at once (a warp's FP64 instruction holds its
 // scheduler's FP64 unit for about 64 cycles on this GPU, so one SM's update bounds a
@@ -418,7 +434,7 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
   const int nr = (kx + kXC - 1) / kXC;               // row slots of a CTA
   double* Srow = xsm;                                 // nr x kx
   double* Lmine = xsm + (size_t)nr * kx;              // nr x kx: L[a][q] of this CTA's rows
-  if (w.qflag[0] != 1) {                              // the same decision in every CTA
+  if (nq > 0 && w.qflag[0] != 1) {                    // the same decision in every CTA
     if (c == 0 && tid == 0) *w.rank = 0;
     return;
   }
@@ -569,10 +585,30 @@ trsm_kernel(const double* __restrict__ Ahat, const double* __restrict__ Mhat, in
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   double* Ls = tsm;                                    // packed columns, r (r - 1) / 2
   double* zs = tsm + (size_t)n * (n - 1) / 2 + (size_t)wid * n;
-  for (int i = wid; i < r; i += kTriWarps) {
-    const double rli = w.rl[i];
-    const int o = col_off(i, r) - i - 1;   // Ls[o + q] for q > i
-    for (int q = i + 1 + lane; q < r; q += 32) Ls[o + q] = w.Lt[i * n + q] * rli;
+  // (two columns of a warp in flight: their loads would otherwise wait one after another)
+  for (int i0 = wid; i0 < r; i0 += 2 * kTriWarps) {
+    double v[2][NS];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = i0 + h * kTriWarps;
+#pragma unroll
+      for (int t = 0; t < NS; ++t) {
+        const int q = lane + 32 * t;
+        v[h][t] = (i < r && q > i && q < r) ? w.Lt[i * n + q] : 0.0;
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = i0 + h * kTriWarps;
+      if (i >= r) continue;
+      const double rli = w.rl[i];
+      const int o = col_off(i, r) - i - 1;   // Ls[o + q] for q > i
+#pragma unroll
+      for (int t = 0; t < NS; ++t) {
+        const int q = lane + 32 * t;
+        if (32 * t + 31 > i && q > i && q < r) Ls[o + q] = v[h][t] * rli;
+      }
+    }
   }
   __syncthreads();
   const int c = blockIdx.x * kTriWarps + wid;
@@ -595,24 +631,7 @@ trsm_kernel(const double* __restrict__ Ahat, const double* __restrict__ Mhat, in
     }
     acc[t] = v;
   }
-  for (int i = 0; i < r; ++i) {
-    const int ti = i >> 5;
-    double a = acc[0];
-#pragma unroll
-    for (int t = 1; t < NS; ++t)
-      if (ti == t) a = acc[t];
-    a = __shfl_sync(0xffffffffu, a, i & 31);
-    if (lane == 0) zs[i] = a;
-    const int o = col_off(i, r) - i - 1;   // Ls[o + q] for q > i
-#pragma unroll
-    for (int t = 0; t < NS; ++t) {
-      if (t >= ti) {
-        const int q = lane + 32 * t;
-        const double l = (q > i && q < r) ? Ls[o + q] : 0.0;
-        acc[t] = fma(-l, a, acc[t]);
-      }
-    }
-  }
+  forward_solve<NS>(Ls, r, lane, acc, zs);
   __syncwarp();
   double* out = pass == 0 ? w.Z : w.T;
   for (int q = lane; q < r; q += 32) out[q * n + c] = zs[q] * w.rl[q];
@@ -635,78 +654,123 @@ __device__ __forceinline__ float start_value(int a, int j, unsigned salt) {
 }
 // Solves per eigenvector (each followed by orthonormalisation inside the clusters).
 constexpr int kInvIters = 3;
+// Exchange of one 8-byte value per row among the CTAs of a cluster without a cluster
+// barrier: a row's warp stores its value into the slot of that row in every CTA
+// (st.async, lane q to CTA q), and the store counts its bytes on that CTA's mbarrier; a CTA's
+// readers wait on their own mbarrier for the bytes of all rows of the step.  The
+// barrier.cluster form has to wait for the acknowledgement of the stores before it arrives:
+// a Householder step took 2.0 us with it, 0.6 us with this.
+__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void push_pair(const void* slot, const void* bar, int rank, unsigned lo, unsigned hi) {
+  unsigned a, m;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(slot)), "r"(rank));
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(m) : "r"(smem_u32(bar)), "r"(rank));
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(a), "r"(lo),
+               "r"(hi), "r"(m)
+               : "memory");
+}
+__device__ __forceinline__ void bar_init(unsigned long long* bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void bar_expect(unsigned long long* bar, unsigned bytes) {
+  asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n" ::"r"(smem_u32(bar)),
+               "r"(bytes)
+               : "memory");
+}
+// Waits for the phase of the given parity; false after about a second (the callers then
+// leave their loops, and the solve reports the result as not finite).
+__device__ __forceinline__ bool bar_wait(unsigned long long* bar, unsigned parity) {
+  const long long t0 = clock64();
+  while (true) {
+    unsigned done;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if (clock64() - t0 > 2000000000LL) return false;
+  }
+}
+
 // Householder tridiagonalisation of sym(T), eigenvalues by multisection of the Sturm
 // count, and the clusters and shifts of the inverse iteration, on a cluster of kEC
-// CTAs (one per SM), so that each Householder step touches kEC times fewer rows per
-// SM: a one-CTA form is bound by the work every warp repeats and by the two passes of
-// the trailing block through one SM's shared memory (about 5400 cycles a step at
-// n = 170).
-// CTA c holds the rows g = c + kEC la of sym(T) (stride ld = 32 NS + 1, columns from r
-// on zero), one warp per row.  The update keeps A exactly symmetric (the two products
-// rounded separately, then added, the same for (g, b) and (b, g)), so row j is column
-// j bit for bit and is read contiguously from its owner.  A step:
-//   every CTA gathers row j from its owner through distributed shared memory and forms
-//   the reflector's scalars and v (all CTAs compute the same values); CTA 0 writes v_j
-//   as row j of the back-transformation's reflector block;
-//   p = t A22 v on the CTA's rows, and the CTA's part of p.v;  cluster barrier;
-//   every CTA gathers p and the kEC parts, forms K and w = p - K v, and updates its
-//   rows;  cluster barrier.
+// CTAs (one per SM).  A step is a chain of dependent operations, so the kernel is built to
+// have few of them and one exchange a step:
+//   CTA c holds the rows g = c + kEC wid of sym(T), one warp a row, the row in registers
+//   (lane l: columns l, l + 32, ...; columns from r on are zero).  The update keeps A
+//   exactly symmetric (the two products rounded separately, then added, the same for
+//   (g, b) and (b, g)), so row j is column j bit for bit.
+//   Step j, in every warp with a row g >= j: it holds row j (x), forms the reflector v and
+//   its scalars by itself, then p_g = t A_g . v, and sends p_g and its element A_g,j+1 of
+//   row j + 1 to all CTAs.  With p and row j + 1 of all rows: K = t/2 p.v, w = p - K v; it
+//   updates its row and the copy of row j + 1, which is the next x.  The warp of row j
+//   records the step (reflector, d_j, e_j) and is done.
+//   The slots are double-buffered by the parity of the step: a warp sends in step j + 2 only
+//   after the values of step j + 1 of every row >= j + 1 have arrived, and the warps of
+//   those rows, the only ones that still read, sent them after they had read step j's.
+// At n = 170 a step takes 0.6 us; with the matrix in shared memory, five CTA barriers and two
+// cluster barriers it took 2.5 us and the kernel 460 us.
 // Then every CTA brackets its share of the eigenvalues by multisection (a warp of 32
 // points per eigenvalue), and CTA 0 gathers them, forms the clusters and shifts of the
-// inverse iteration and writes the tridiagonal matrix.  A CTA's shared memory is read
-// by the others only between barriers that every thread of every CTA passes the same
-// number of times (no branch around a barrier depends on anything but n, r and data
-// that all CTAs hold identically).
+// inverse iteration and writes the tridiagonal matrix.  Every thread of every CTA passes the
+// same number of cluster barriers.
 constexpr int kEC = 8;
-constexpr int kEThreads = 1024;
 template <int NS>
-__global__ void __cluster_dims__(kEC, 1, 1) __launch_bounds__(kEThreads)
+__global__ void __cluster_dims__(kEC, 1, 1) __launch_bounds__(32 * 32 * NS / kEC)
 eig32_cl_kernel(int n, DW w) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
-  constexpr int ld = 32 * NS + 1;
-  constexpr int RW = (32 * NS + kEC - 1) / kEC;       // row slots of a CTA (<= 32)
-  static_assert(RW <= kEThreads / 32, "one warp per row");
-  extern __shared__ float fsm[];
-  float* A = fsm;                                     // RW x ld: rows c + kEC la
-  __shared__ float d[kMaxN], e[kMaxN], e2[kMaxN], tau[kMaxN], xv[kMaxN], vb[kMaxN], pv[kMaxN], wv[kMaxN],
-      lam[kMaxN];
-  __shared__ float wpart[32], s_pd, slo[32], shi[32];
+  constexpr int nwarps = 32 * NS / kEC;               // rows of a CTA, one warp each
+  constexpr int kThreads = 32 * nwarps;
+  __shared__ __align__(16) float2 buf[2][32 * NS];    // p_g and A_g,j+1 of every row
+  __shared__ __align__(8) unsigned long long bars[2];
+  __shared__ float d[kMaxN], e[kMaxN], e2[kMaxN], vb[kMaxN], lam[kMaxN];
+  __shared__ float slo[32], shi[32];
   const int c = (int)cl.block_rank();
   const int r = *w.rank;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  constexpr int nwarps = kEThreads / 32;
-  // this CTA's rows of sym(T) in FP32, read before any CTA writes sym(T) back
-  for (int q = tid; q < RW * ld; q += kEThreads) {
-    const int la = q / ld, b = q - la * ld, g = c + kEC * la;
-    A[q] = (g < r && b < r) ? (float)(0.5 * (w.T[g * n + b] + w.T[b * n + g])) : 0.f;
+  const int g = c + kEC * wid;                        // this warp's row
+  // its row and row 0 of sym(T) in FP32, read before any CTA writes sym(T) back
+  float A[NS], x[NS];
+#pragma unroll
+  for (int i = 0; i < NS; ++i) {
+    const int b = lane + 32 * i;
+    A[i] = (g < r && b < r) ? (float)(0.5 * (w.T[g * n + b] + w.T[b * n + g])) : 0.f;
+    x[i] = b < r ? (float)(0.5 * (w.T[b] + w.T[b * n])) : 0.f;
   }
-  for (int b = tid; b < kMaxN; b += kEThreads) pv[b] = 0.f;
+  for (int b = tid; b < 64 * NS; b += kThreads) (&buf[0][0])[b] = make_float2(0.f, 0.f);
+  if (tid == 0) {
+    bar_init(&bars[0]);
+    bar_init(&bars[1]);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
   cl.sync();
-  // sym(T) back into T for the FP64 refinement: the pairs b >= g of this CTA's rows
-  // (each pair read and written by its one owner)
-  for (int la = wid; la < RW; la += nwarps) {
-    const int g = c + kEC * la;
-    if (g >= r) continue;
+  // sym(T) back into T for the FP64 refinement: the pairs b >= g of this warp's row (each
+  // pair read and written by its one owner)
+  if (g < r)
     for (int b = g + lane; b < r; b += 32) {
       const double v = 0.5 * (w.T[g * n + b] + w.T[b * n + g]);
       w.T[g * n + b] = v;
       w.T[b * n + g] = v;
     }
-  }
   float* V = w.A32;                                   // reflector rows for backtr_kernel
-  __shared__ float pdv[kEC];
-  for (int j = 0; j + 2 < r; ++j) {
-    const int j1 = j + 1;
-    {                                                   // row j (= column j) from its owner
-      const float* rowj = cl.map_shared_rank(A, j % kEC) + (j / kEC) * ld;
-      for (int b = tid; b < r; b += kEThreads) xv[b] = rowj[b];
+  float *gd = w.T3, *ge = w.T3 + n;                   // d and e, by the warps of their rows
+  const bool arms = g < r && g + kEC >= r;            // the CTA's last row: its warp leaves last
+  bool ok = true;
+  for (int j = 0; j + 2 < r && j <= g && g < r; ++j) {
+    const int j1 = j + 1, par = j & 1;
+    if (arms && lane == 0) bar_expect(&bars[par], 8u * (unsigned)(r - j));
+    float part = 0.f, a0s = 0.f, a1s = 0.f;
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      if (lane + 32 * i > j1) part = fmaf(x[i], x[i], part);
+      if (i == (j1 >> 5)) { a0s = x[i]; a1s = A[i]; }
     }
-    __syncthreads();
-    float part = 0.f;
-    for (int b = j + 2 + lane; b < r; b += 32) part = fmaf(xv[b], xv[b], part);
+    const float a0 = __shfl_sync(0xffffffffu, a0s, j1 & 31);
+    const float a1 = __shfl_sync(0xffffffffu, a1s, j1 & 31);   // A_g,j+1
     const float xn2 = warp_sumf(part);
-    const float a0 = xv[j1];
     float beta = a0, t = 0.f, scale = 0.f;
     if (xn2 > 0.f) {
       // hardware approximations (a few ulps): the reflector stays orthogonal to FP32
@@ -716,84 +780,81 @@ eig32_cl_kernel(int n, DW w) {
       t = __fdividef(beta - a0, beta);
       scale = __fdividef(1.f, a0 - beta);
     }
-    if (tid == 0) { d[j] = xv[j]; e[j] = beta; tau[j] = t; }
-    for (int b = tid; b < 32 * NS; b += kEThreads)
-      vb[b] = (b == j1) ? 1.f : ((b > j1 && b < r) ? xv[b] * scale : 0.f);
-    __syncthreads();
-    if (c == 0)                                         // v_j (1 at j + 1, 0 above; 0 when t = 0)
-      for (int b = tid; b < r; b += kEThreads) V[j * r + b] = (t != 0.f) ? vb[b] : 0.f;
-    // p = t A22 v on this CTA's rows, and the CTA's part of p.v
-    float pd = 0.f;
-    if (wid < RW && t != 0.f) {
-      const int g = c + kEC * wid;
-      if (g >= j1 && g < r) {                           // warp-uniform
-        const float* Ar = A + wid * ld + lane;
-        float s = 0.f;
+    float v[NS], s = 0.f;
 #pragma unroll
-        for (int i = 0; i < NS; ++i) s = fmaf(Ar[32 * i], vb[lane + 32 * i], s);
-        s = warp_sumf(s);
-        const float p = t * s;
-        if (lane == 0) pv[g] = p;
-        pd = p * vb[g];
+    for (int i = 0; i < NS; ++i) {
+      const int b = lane + 32 * i;
+      v[i] = b == j1 ? 1.f : (b > j1 ? x[i] * scale : 0.f);
+      s = fmaf(A[i], v[i], s);
+    }
+    s = warp_sumf(s);
+    if (lane < kEC) push_pair(&buf[par][g], &bars[par], lane, __float_as_uint(t * s), __float_as_uint(a1));
+    if (g == j) {
+      // this row's step: the reflector and the tridiagonal entries; no one reads this row again
+#pragma unroll
+      for (int i = 0; i < NS; ++i) {
+        const int b = lane + 32 * i;
+        if (b < r) V[j * r + b] = (t != 0.f) ? v[i] : 0.f;
+        if (b == j) gd[j] = x[i];
       }
-    }
-    if (lane == 0) wpart[wid] = pd;
-    __syncthreads();
-    if (wid == 0) {
-      const float q = warp_sumf(wpart[lane]);
-      if (lane == 0) s_pd = q;
-    }
-    cl.sync();                                          // p and the parts of p.v complete
-    if (tid < kEC) pdv[tid] = *cl.map_shared_rank(&s_pd, tid);
-    __syncthreads();
-    float kk = 0.f;                                     // K = (t/2) p.v, parts in CTA order
-#pragma unroll
-    for (int q = 0; q < kEC; ++q) kk += pdv[q];
-    kk *= 0.5f * t;
-    for (int b = tid; b < 32 * NS; b += kEThreads) {
-      const float pb = (t != 0.f && b >= j1 && b < r) ? *cl.map_shared_rank(&pv[b], b % kEC) : 0.f;
-      wv[b] = fmaf(-kk, vb[b], pb);                     // w = p - K v (0 outside the trailing block)
-    }
-    __syncthreads();
-    // A22 -= v w^T + w v^T on this CTA's rows; the two products rounded alone and then
-    // added, so that (g, b) and (b, g) get the same value
-    if (wid < RW && t != 0.f) {
-      const int g = c + kEC * wid;
-      if (g >= j1 && g < r) {
-        float* Ar = A + wid * ld + lane;
-        const float vg = vb[g], wg = wv[g];
-#pragma unroll
-        for (int i = 0; i < NS; ++i) {
-          const int b = lane + 32 * i;
-          Ar[32 * i] = Ar[32 * i] - __fadd_rn(__fmul_rn(vg, wv[b]), __fmul_rn(wg, vb[b]));
-        }
+      if (lane == 0) {
+        ge[j] = beta;
+        V[r * r + j] = t;
       }
+      break;
     }
-    cl.sync();                                          // rows updated before the next gather
-  }
-  if (tid == 0) {
-    if (r >= 2) {
-      const float* ra = cl.map_shared_rank(A, (r - 2) % kEC) + ((r - 2) / kEC) * ld;
-      const float* rb = cl.map_shared_rank(A, (r - 1) % kEC) + ((r - 1) / kEC) * ld;
-      d[r - 2] = ra[r - 2];
-      e[r - 2] = rb[r - 2];
-      tau[r - 2] = 0.f;
+    float vgs = 0.f;
+#pragma unroll
+    for (int i = 0; i < NS; ++i)
+      if (i == (g >> 5)) vgs = v[i];
+    const float vg = __shfl_sync(0xffffffffu, vgs, g & 31);
+    ok = bar_wait(&bars[par], (unsigned)(j >> 1) & 1u);
+    if (!__all_sync(0xffffffffu, ok)) {
+      ok = false;
+      break;
     }
-    if (r >= 1) {
-      const float* rb = cl.map_shared_rank(A, (r - 1) % kEC) + ((r - 1) / kEC) * ld;
-      d[r - 1] = rb[r - 1];
-      e[r - 1] = 0.f;
-      tau[r - 1] = 0.f;
+    float pw[NS], old[NS], pd = 0.f;
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      const int b = lane + 32 * i;
+      const float2 q = buf[par][b];
+      pw[i] = (b >= j1 && b < r) ? q.x : 0.f;
+      old[i] = q.y;
+      pd = fmaf(pw[i], v[i], pd);
+    }
+    const float pg = buf[par][g].x, p1 = buf[par][j1].x;
+    const float kk = 0.5f * t * warp_sumf(pd);
+    const float wg = fmaf(-kk, vg, pg), w1 = fmaf(-kk, 1.f, p1);
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      const float wi = fmaf(-kk, v[i], pw[i]);        // w = p - K v (0 outside the trailing block)
+      x[i] = t != 0.f ? old[i] - __fadd_rn(wi, __fmul_rn(w1, v[i])) : old[i];
+      if (t != 0.f) A[i] = A[i] - __fadd_rn(__fmul_rn(vg, wi), __fmul_rn(wg, v[i]));
     }
   }
-  if (c == 0) {                                         // the rows without a reflector, and tau
-    for (int q = max(0, r - 2) * r + tid; q < r * r; q += kEThreads) V[q] = 0.f;
-    for (int j = tid; j < r; j += kEThreads) V[r * r + j] = (j + 2 < r) ? tau[j] : 0.f;
+  // the last entries: rows r - 2 and r - 1 hold them
+  if (g < r && g + 2 >= r) {
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      const int b = lane + 32 * i;
+      if (b == g) gd[g] = ok ? A[i] : __int_as_float(0x7fffffff);
+      if (g + 2 == r && b == r - 1) ge[g] = A[i];
+      if (b < r) V[g * r + b] = 0.f;                    // no reflector
+    }
+    if (lane == 0) {
+      if (g + 1 == r) ge[g] = 0.f;
+      V[r * r + g] = 0.f;
+    }
+  }
+  cl.sync();                                            // d and e complete; no more sends
+  for (int b = tid; b < r; b += kThreads) {
+    d[b] = __ldcg(gd + b);
+    e[b] = __ldcg(ge + b);
   }
   __syncthreads();
   // --- Gershgorin interval (every CTA, the same values)
   float lo = 3.4e38f, hi = -3.4e38f;
-  for (int i = tid; i < r; i += kEThreads) {
+  for (int i = tid; i < r; i += kThreads) {
     const float rad = fabsf(e[i]) + (i > 0 ? fabsf(e[i - 1]) : 0.f);
     lo = fminf(lo, d[i] - rad);
     hi = fmaxf(hi, d[i] + rad);
@@ -811,45 +872,42 @@ eig32_cl_kernel(int n, DW w) {
   const float span = fmaxf(fmaxf(fabsf(lo), fabsf(hi)), 1e-30f);
   const float pivmin = 1e-30f * fmaxf(span * span, 1.f);
   // --- eigenvalues by multisection of the Sturm count, CTA c taking the eigenvalues
-  // [c qn, (c + 1) qn): a group of 8 lanes brackets one eigenvalue; each lane counts
-  // the eigenvalues below one of 8 interior points of the group's interval, which
-  // splits it into 9 parts; 8 rounds shrink the Gershgorin interval by 9^8 = 4.3e7, to
-  // the FP32 resolution of the spectrum (eigenvalues near 0 need no more: the
-  // refinement takes them to FP64).
+  // [c qn, (c + 1) qn), a warp one eigenvalue: each lane counts the eigenvalues below one of
+  // 32 interior points of the interval, which splits it into 33 parts; 5 rounds shrink the
+  // Gershgorin interval by 33^5 = 3.9e7, to the FP32 resolution of the spectrum
+  // (eigenvalues near 0 need no more: the refinement takes them to FP64).  A round is a
+  // chain of r dependent divisions, so wide splits beat more rounds (8 rounds of 9 parts
+  // took 1.6 times as long).
   const int qn = (r + kEC - 1) / kEC, i0 = c * qn, i1 = min(r, i0 + qn);
-  {
-    const int grp = tid >> 3, sl = tid & 7;
-    const int gsh = lane & 24;
-    const float frac = (float)(sl + 1) * (1.0f / 9.0f);
-    if (i0 + 4 * wid < i1) {                            // warp-uniform
-      const int i = min(i0 + grp, i1 - 1);
-      float a = lo - 1e-6f * span, b = hi + 1e-6f * span;
-      for (int round = 0; round < 8; ++round) {
-        const float wd = b - a;
-        const float x = fmaf(wd, frac, a);
-        int cnt = 0;
-        float q = d[0] - x;
+  if (i0 + wid < i1) {                                  // warp-uniform
+    const int i = i0 + wid;
+    const float frac = (float)(lane + 1) * (1.0f / 33.0f);
+    float a = lo - 1e-6f * span, b = hi + 1e-6f * span;
+    for (int round = 0; round < 5; ++round) {
+      const float wd = b - a;
+      const float xx = fmaf(wd, frac, a);
+      int cnt = 0;
+      float q = d[0] - xx;
+      if (fabsf(q) < pivmin) q = -pivmin;
+      cnt += q < 0.f;
+      for (int jj = 1; jj < r; ++jj) {
+        q = (d[jj] - xx) - __fdividef(e2[jj - 1], q);
         if (fabsf(q) < pivmin) q = -pivmin;
         cnt += q < 0.f;
-        for (int jj = 1; jj < r; ++jj) {
-          q = (d[jj] - x) - __fdividef(e2[jj - 1], q);
-          if (fabsf(q) < pivmin) q = -pivmin;
-          cnt += q < 0.f;
-        }
-        // counts grow with x: the first point with more than i eigenvalues below it
-        const unsigned m = (__ballot_sync(0xffffffffu, cnt > i) >> gsh) & 0xffu;
-        const int first = m ? __ffs(m) - 1 : 8;
-        const float na = (first == 0) ? a : fmaf(wd, (float)first * (1.0f / 9.0f), a);
-        const float nb = (first == 8) ? b : fmaf(wd, (float)(first + 1) * (1.0f / 9.0f), a);
-        a = na;
-        b = nb;
       }
-      if (sl == 0 && i0 + grp < i1) lam[i] = 0.5f * (a + b);
+      // counts grow with x: the first point with more than i eigenvalues below it
+      const unsigned m = __ballot_sync(0xffffffffu, cnt > i);
+      const int first = m ? __ffs(m) - 1 : 32;
+      const float na = (first == 0) ? a : fmaf(wd, (float)first * (1.0f / 33.0f), a);
+      const float nb = (first == 32) ? b : fmaf(wd, (float)(first + 1) * (1.0f / 33.0f), a);
+      a = na;
+      b = nb;
     }
+    if (lane == 0) lam[i] = 0.5f * (a + b);
   }
   cl.sync();                                            // every CTA's eigenvalues bracketed
   if (c == 0)
-    for (int i = tid; i < r; i += kEThreads)
+    for (int i = tid; i < r; i += kThreads)
       if (i >= qn) lam[i] = *cl.map_shared_rank(&lam[i], i / qn);
   cl.sync();                                            // CTA 0 has read the others' eigenvalues
   if (c != 0) return;
@@ -880,7 +938,7 @@ eig32_cl_kernel(int n, DW w) {
     s_ncl = nc;
   }
   __syncthreads();
-  for (int i = tid; i < r; i += kEThreads) {
+  for (int i = tid; i < r; i += kThreads) {
     w.T3[i] = d[i];
     w.T3[n + i] = e[i];
     w.T3[2 * n + i] = shift[i];
@@ -889,7 +947,7 @@ eig32_cl_kernel(int n, DW w) {
     w.T3[3 * n] = tiny;
     w.cls[0] = s_ncl;
   }
-  for (int q = tid; q <= s_ncl; q += kEThreads) w.cls[1 + q] = cst[q];
+  for (int q = tid; q <= s_ncl; q += kThreads) w.cls[1 + q] = cst[q];
 }
 
 // ------------------------------------- 3a. inverse iteration (one CTA per cluster) --
@@ -1631,10 +1689,29 @@ backsub_kernel(int n, int k, DW w, double* __restrict__ Y) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   double* Lr = tsm;                                    // packed rows, r (r - 1) / 2
   double* zs = tsm + (size_t)n * (n - 1) / 2 + (size_t)wid * n;
-  for (int i = 1 + wid; i < r; i += kTriWarps) {
-    const double rli = w.rl[i];
-    double* dst = Lr + i * (i - 1) / 2;
-    for (int q = lane; q < i; q += 32) dst[q] = w.L[i * n + q] * rli;
+  for (int i0 = 1 + wid; i0 < r; i0 += 2 * kTriWarps) {   // two rows of a warp in flight
+    double v[2][NS];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = i0 + h * kTriWarps;
+#pragma unroll
+      for (int t = 0; t < NS; ++t) {
+        const int q = lane + 32 * t;
+        v[h][t] = (i < r && q < i) ? w.L[i * n + q] : 0.0;
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = i0 + h * kTriWarps;
+      if (i >= r) continue;
+      const double rli = w.rl[i];
+      double* dst = Lr + i * (i - 1) / 2;
+#pragma unroll
+      for (int t = 0; t < NS; ++t) {
+        const int q = lane + 32 * t;
+        if (32 * t < i && q < i) dst[q] = v[h][t] * rli;
+      }
+    }
   }
   __syncthreads();
   const int c = blockIdx.x * kTriWarps + wid;
@@ -1646,24 +1723,7 @@ backsub_kernel(int n, int k, DW w, double* __restrict__ Y) {
     const int q = lane + 32 * t;
     acc[t] = (q < r) ? w.W[q * n + oc] : 0.0;
   }
-  for (int i = r - 1; i >= 0; --i) {
-    const int ti = i >> 5;
-    double a = acc[0];
-#pragma unroll
-    for (int t = 1; t < NS; ++t)
-      if (ti == t) a = acc[t];
-    a = __shfl_sync(0xffffffffu, a, i & 31);
-    if (lane == 0) zs[i] = a;
-    const double* li = Lr + i * (i - 1) / 2;        // li[q] for q < i
-#pragma unroll
-    for (int t = 0; t < NS; ++t) {
-      if (t <= ti) {
-        const int q = lane + 32 * t;
-        const double l = (q < i) ? li[q] : 0.0;
-        acc[t] = fma(-l, a, acc[t]);
-      }
-    }
-  }
+  backward_solve<NS>(Lr, r, lane, acc, zs);
   __syncwarp();
   const int* perm = w.perm;
   for (int i = lane; i < n; i += 32) {
@@ -1749,12 +1809,10 @@ void trsm(const double* Ahat, const double* Mhat, int n, double sigma, int pass,
     default: trsm_ns<kRowsPerLane>(Ahat, Mhat, n, sigma, pass, w, s); break;
   }
 }
-// FP32 eigensolve launch: each CTA of the cluster holds its rows of T (stride 32 NS + 1).
+// FP32 eigensolve launch: a warp per row, n <= 32 NS rows over the cluster.
 template <int NS>
 void eig32(int n, const DW& w, cudaStream_t s) {
-  const size_t esm = (size_t)((32 * NS + kEC - 1) / kEC) * (32 * NS + 1) * sizeof(float);
-  BMG_CUDA(cudaFuncSetAttribute(eig32_cl_kernel<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)esm));
-  eig32_cl_kernel<NS><<<kEC, kEThreads, esm, s>>>(n, w);
+  eig32_cl_kernel<NS><<<kEC, 32 * 32 * NS / kEC, 0, s>>>(n, w);
   check_launch("eig32_cl_kernel");
 }
 void backsub(int n, int k, const DW& w, double* Y, cudaStream_t s) {
@@ -1784,10 +1842,11 @@ void dense_eig(const double* Ahat, const double* Mhat, int n, double sigma, int 
   TraceRange trace("enriched eigensolve");
   prof_begin(KC_DENSE, s);
   DW w = carve(work, n);
-  // 1. basis: whole pivoted factorisation, or the block form when the leading nq x nq
-  //    block repeats (its factor cached in the workspace)
-  if (nq > 0 && nq <= kMaxQ && nq < n && (size_t)(n - nq) * (n - nq) * sizeof(double) <= 200 * 1024) {
-    const int kx = n - nq;
+  // 1. basis: the block form, with the leading nq x nq block's factor cached in the
+  //    workspace when it repeats, else (nq = 0) the whole matrix as the new block
+  if (nq < 0 || nq > kMaxQ || nq >= n) nq = 0;
+  const int kx = n - nq;
+  if (nq > 0) {
     qfactor_kernel<kFactorWarps><<<1, kFactorWarps * 32, 0, s>>>(Mhat, n, nq, w, drop_tol);
     check_launch("qfactor_kernel");
     const size_t xsm = sizeof(double) * ((size_t)nq * (nq - 1) / 2 + (size_t)kTriWarps * nq);
@@ -1797,20 +1856,17 @@ void dense_eig(const double* Ahat, const double* Mhat, int n, double sigma, int 
       xsolve_kernel<2><<<(kx + kTriWarps - 1) / kTriWarps, kTriWarps * 32, xsm, s>>>(Mhat, n, nq, kx, w);
     }
     check_launch("xsolve_kernel");
-    const int nt = (kx + 7) / 8;
-    schur_kernel<<<dim3(nt, nt), 64, 0, s>>>(Mhat, n, nq, kx, w);
-    check_launch("schur_kernel");
-    const size_t xfs = 2 * (size_t)((kx + kXC - 1) / kXC) * kx * sizeof(double);
-    BMG_CUDA(cudaFuncSetAttribute(xfactor_cl_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xfs));
-    xfactor_cl_kernel<<<kXC, kXThreads, xfs, s>>>(n, nq, kx, w, drop_tol);
-    check_launch("xfactor_cl_kernel");
   } else {
-    const size_t smemS = (size_t)n * n * sizeof(double);
-    const bool useS = smemS <= 200 * 1024;
-    if (useS) BMG_CUDA(cudaFuncSetAttribute(basis_kernel<kBasisWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smemS));
-    basis_kernel<kBasisWarps><<<1, kBasisWarps * 32, useS ? smemS : 0, s>>>(Mhat, n, w, useS ? 1 : 0, drop_tol);
-    check_launch("basis_kernel");
+    scaling_kernel<<<(n + 127) / 128, 128, 0, s>>>(Mhat, n, w);
+    check_launch("scaling_kernel");
   }
+  const int nt = (kx + 7) / 8;
+  schur_kernel<<<dim3(nt, nt), 64, 0, s>>>(Mhat, n, nq, kx, w);
+  check_launch("schur_kernel");
+  const size_t xfs = 2 * (size_t)((kx + kXC - 1) / kXC) * kx * sizeof(double);
+  BMG_CUDA(cudaFuncSetAttribute(xfactor_cl_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xfs));
+  xfactor_cl_kernel<<<kXC, kXThreads, xfs, s>>>(n, nq, kx, w, drop_tol);
+  check_launch("xfactor_cl_kernel");
   // 2. reduced standard matrix
   trsm(Ahat, Mhat, n, sigma, 0, w, s);
   trsm(Ahat, Mhat, n, sigma, 1, w, s);
