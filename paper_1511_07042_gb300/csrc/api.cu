@@ -423,6 +423,19 @@ static const double* opDA_or_compute(const bmg_problem* p, int f, int j) {
   return nullptr;
 }
 
+// nu Jacobi sweeps on X, which alternate between X and work and end in X: an odd count
+// starts from a copy (a copy after every sweep took as long as a third of the sweep).
+template <typename T>
+static void jacobi_sweeps(const Mesh& m, const T* a, const T* mm, const T* da, const T* dm, T* X, const T* B,
+                          const T* sft, int ld, int nu, double omega, T* work, cudaStream_t s) {
+  T *src = X, *dst = work;
+  if (nu % 2 == 1) {
+    BMG_CUDA(cudaMemcpyAsync(work, X, sizeof(T) * (size_t)m.n * ld, cudaMemcpyDeviceToDevice, s));
+    std::swap(src, dst);
+  }
+  for (int it = 0; it < nu; ++it, std::swap(src, dst)) jacobi_sweep<T>(m, a, mm, da, dm, src, dst, B, sft, ld, omega, s);
+}
+
 extern "C" bmg_status bmg_spmm(const bmg_problem* p, int f, int level, const double* X, int k, int ld,
                                double* AX, double* MX, void* stream) {
   return guarded([&] {
@@ -446,10 +459,7 @@ extern "C" bmg_status bmg_smooth(const bmg_problem* p, int f, int level, double*
     (void)opDA_or_compute;
     if (smoother == BMG_SMOOTH_JACOBI) {
       if (!work) fail(BMG_ERR_INVALID_ARG, "Jacobi needs a work block");
-      for (int it = 0; it < nu; ++it) {
-        jacobi_sweep(m, a, mm, da, dm, X, work, B, sft, ld, omega, s);
-        BMG_CUDA(cudaMemcpyAsync(X, work, sizeof(double) * (size_t)m.n * ld, cudaMemcpyDeviceToDevice, s));
-      }
+      jacobi_sweeps<double>(m, a, mm, da, dm, X, B, sft, ld, nu, omega, work, s);
     } else if (smoother == BMG_SMOOTH_MCGS || smoother == BMG_SMOOTH_MCSGS) {
       const Level& lv = p->lev[level];
       for (int it = 0; it < nu; ++it) {
@@ -1552,10 +1562,7 @@ extern "C" bmg_status bmg_smooth_f32(bmg_problem* p, int f, int level, float* X,
     const float *da = Ops<float>::DA(p, f, level), *dm = Ops<float>::DM(p, f, level);
     if (smoother == BMG_SMOOTH_JACOBI) {
       if (!work) fail(BMG_ERR_INVALID_ARG, "Jacobi needs a work block");
-      for (int it = 0; it < nu; ++it) {
-        jacobi_sweep<float>(m, a, mm, da, dm, X, work, B, sft, ld, omega, s);
-        BMG_CUDA(cudaMemcpyAsync(X, work, sizeof(float) * (size_t)m.n * ld, cudaMemcpyDeviceToDevice, s));
-      }
+      jacobi_sweeps<float>(m, a, mm, da, dm, X, B, sft, ld, nu, omega, work, s);
     } else if (smoother == BMG_SMOOTH_MCGS || smoother == BMG_SMOOTH_MCSGS) {
       const Level& lv = p->lev[level];
       for (int it = 0; it < nu; ++it) {
