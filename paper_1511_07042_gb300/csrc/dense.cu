@@ -68,6 +68,13 @@ __device__ __forceinline__ double rcp_nr(double x) {
   const double y = (double)(1.0f / (float)x);
   return y * fma(-x, y, 2.0);
 }
+// 1/x to float64 accuracy for x in the FP32 normal range: FP32 seed and one step of third
+// order, y (1 + e + e^2) with e = 1 - x y.
+__device__ __forceinline__ double rcp_full(double x) {
+  const double y = (double)(1.0f / (float)x);
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
 __device__ __forceinline__ float warp_sumf(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -397,123 +404,202 @@ schur_kernel(const double* __restrict__ Mhat, int n, int nq, int kx, DW w) {
   w.S[b * kx + a] = v;
 }
 
+// Exchange of one 8-byte value per row among the CTAs of a cluster without a cluster
+// barrier: a row's warp stores its value into the slot of that row in every CTA
+// (st.async, lane q to CTA q), and the store counts its bytes on that CTA's mbarrier; a CTA's
+// readers wait on their own mbarrier for the bytes of all rows of the step.  The
+// barrier.cluster form has to wait for the acknowledgement of the stores before it arrives:
+// a Householder step took 2.0 us with it, 0.6 us with this.
+__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void push_pair(const void* slot, const void* bar, int rank, unsigned lo, unsigned hi) {
+  unsigned a, m;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(slot)), "r"(rank));
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(m) : "r"(smem_u32(bar)), "r"(rank));
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(a), "r"(lo),
+               "r"(hi), "r"(m)
+               : "memory");
+}
+__device__ __forceinline__ void bar_init(unsigned long long* bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void bar_expect(unsigned long long* bar, unsigned bytes) {
+  asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n" ::"r"(smem_u32(bar)),
+               "r"(bytes)
+               : "memory");
+}
+// Waits for the phase of the given parity; false after about a second (the callers then
+// leave their loops, and the solve reports the result as not finite).
+__device__ __forceinline__ bool bar_wait(unsigned long long* bar, unsigned parity) {
+  const long long t0 = clock64();
+  while (true) {
+    unsigned done;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if (clock64() - t0 > 2000000000LL) return false;
+  }
+}
+
 // Pivoted Cholesky of S_X and assembly of the factor of the whole of M-hat in the
 // layout of the solves below (L: row i holds L[i][0..i] in pivot order; Lt: row q holds
 // column q of L; rl, perm, d, rank).  A deficient M_Q gives rank 0.
 // The factorisation runs on a cluster of kXC CTAs, one per SM: the update, the bulk of
 // the FP64 work, then runs on kXC SMs at once (a warp's FP64 instruction holds its
-// scheduler's FP64 unit for about 64 cycles on this GPU, so one SM's update bounds a
-// one-CTA factorisation).  CTA c holds the full rows a = c + kXC la of S_X and the
-// factor entries of those rows.  Pivoting is logical: an eliminated index keeps its
-// row and is only marked, and the pivot order is assembled at the end.  A step: each
-// CTA's largest remaining diagonal into its candidate slot (double-buffered by step
-// parity, so that a CTA a step ahead never overwrites a slot still being read); one
-// cluster barrier; every CTA reads the kXC candidates through distributed shared memory
-// and takes the same pivot p (largest key, then smallest index), stages row p of its
-// owner while warp 0 forms 1/sqrt(piv), and updates its own remaining rows (each
-// element gets the fused multiply-adds of the unblocked right-looking algorithm, in
-// pivot order).  Row p is never written again once chosen, so the other CTAs may read
-// it while its owner moves on.
+// scheduler's FP64 unit for 64 cycles).  CTA c holds the rows a = c + kXC wid of S_X, one
+// warp a row, the row in registers (lane l: columns l, l + 32, ...), and one more warp for
+// the pivots' reciprocals.  Pivoting is logical: an eliminated index keeps its row and is
+// only marked, and the pivot order is assembled at the end.  A step is two exchanges:
+//   every remaining row sends its diagonal to all CTAs; every warp takes the same pivot p
+//   (largest key, then smallest index);
+//   every remaining row sends its element r_a of column p, while the extra warp of each CTA
+//   forms 1/piv; then row a subtracts (r_a / piv) r_b.
+// The unscaled r_a are kept and scaled by 1/sqrt(piv) at the end.  The buffers alternate with
+// the parity of the step, as in the tridiagonalisation below: a row sends in step j + 2 only
+// after all rows that remain in step j + 1 have sent there, and these, the only ones that
+// still read step j's values, had read them before.
+// At k = 128 a step took 2.3 us with the pivot row fetched between CTA and cluster barriers.
 constexpr int kXC = 8;
-constexpr int kXThreads = 256;
-__global__ void __cluster_dims__(kXC, 1, 1) __launch_bounds__(kXThreads)
+template <int NS>
+__global__ void __cluster_dims__(kXC, 1, 1) __launch_bounds__(32 * (32 * NS / kXC + 1))
 xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
+  constexpr int nrow = 32 * NS / kXC;                 // rows of a CTA, one warp each
+  constexpr int nwarps = nrow + 1, kXThreads = 32 * nwarps;
   extern __shared__ double xsm[];
-  __shared__ double lrow[kMaxN], rls[kMaxN];
+  double* Lmine = xsm;                                // nrow x kx: r_a of each step of this CTA's rows
+  __shared__ __align__(16) double kbuf[2][32 * NS], rbuf[2][32 * NS + 1];   // rbuf's last: 1/piv
+  __shared__ __align__(8) unsigned long long kbar[2], rbar[2];
+  __shared__ double rls[kMaxN];
   __shared__ int perm[kMaxN], pos[kMaxN];
   __shared__ unsigned char done[kMaxN];
-  __shared__ unsigned long long candk[2];
-  __shared__ int candi[2];
-  __shared__ int s_p, s_go;
-  __shared__ double s_piv, s_rl;
   const int c = (int)cl.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  constexpr int nwarps = kXThreads / 32;
-  const int nr = (kx + kXC - 1) / kXC;               // row slots of a CTA
-  double* Srow = xsm;                                 // nr x kx
-  double* Lmine = xsm + (size_t)nr * kx;              // nr x kx: L[a][q] of this CTA's rows
   if (nq > 0 && w.qflag[0] != 1) {                    // the same decision in every CTA
     if (c == 0 && tid == 0) *w.rank = 0;
     return;
   }
-  for (int q = tid; q < nr * kx; q += kXThreads) {
-    const int la = q / kx, a = c + kXC * la;
-    Srow[q] = (a < kx) ? __ldcg(w.S + a * kx + (q - la * kx)) : 0.0;
-    Lmine[q] = 0.0;
+  // pivot order and values through global memory: gperm[j], gpiv[j], then the rank
+  int* gperm = w.srt;
+  int* grank = w.cl;                                  // [0] rank, [1] a wait expired
+  double* gpiv = w.lam;
+  const bool scalar = wid == nrow;
+  const int a = scalar ? kx : c + kXC * wid;          // this warp's row
+  const bool has = a < kx;
+  double S[NS];
+#pragma unroll
+  for (int i = 0; i < NS; ++i) {
+    const int b = lane + 32 * i;
+    S[i] = (has && b < kx) ? __ldcg(w.S + a * kx + b) : 0.0;
   }
+  for (int q = tid; q < nrow * kx; q += kXThreads) Lmine[q] = 0.0;
+  if (tid == 0) {
+    for (int q = 0; q < 2; ++q) { bar_init(&kbar[q]); bar_init(&rbar[q]); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (c == 0) { grank[0] = kx; grank[1] = 0; }
+  }
+  cl.sync();
+  unsigned gone = 0u;                                 // eliminated columns of this lane, a bit per slot
+  // Rows of this CTA still to eliminate.  The extra warp works while there are two: one of
+  // them then remains, whose next values wait for the extra warp's, so that no buffer is
+  // written again before the extra warp has read it.  The last row does its work itself.
+  int mine = c < kx ? (kx - c + kXC - 1) / kXC : 0;
+  bool expired = false;
+  for (int j = 0; j < kx && (has || (scalar && mine > 1)); ++j) {
+    const bool solo = mine == 1;
+    const int par = j & 1;
+    const unsigned ph = (unsigned)(j >> 1) & 1u;
+    if ((scalar || solo) && lane == 0) {
+      bar_expect(&kbar[par], 8u * (unsigned)(kx - j));
+      bar_expect(&rbar[par], 8u * (unsigned)(kx - j) + (solo ? 0u : 8u));
+    }
+    if (!scalar) {
+      double ds = 0.0;
+#pragma unroll
+      for (int i = 0; i < NS; ++i)
+        if (i == (a >> 5)) ds = S[i];
+      ds = __shfl_sync(0xffffffffu, ds, a & 31);
+      if (lane < kXC)
+        push_pair(&kbuf[par][a], &kbar[par], lane, (unsigned)__double2loint(ds), (unsigned)__double2hiint(ds));
+    }
+    expired = !bar_wait(&kbar[par], ph);
+    if (__any_sync(0xffffffffu, expired)) { expired = true; break; }
+    // the pivot: largest key, then smallest index
+    unsigned khi[NS], klo[NS], m1 = 0u;
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      const int b = lane + 32 * i;
+      const unsigned long long key = (b < kx && !((gone >> i) & 1u)) ? pivot_key(kbuf[par][b]) : 0ull;
+      khi[i] = (unsigned)(key >> 32);
+      klo[i] = (unsigned)key;
+      m1 = max(m1, khi[i]);
+    }
+    m1 = __reduce_max_sync(0xffffffffu, m1);
+    unsigned m0 = 0u;
+#pragma unroll
+    for (int i = 0; i < NS; ++i)
+      if (khi[i] == m1) m0 = max(m0, klo[i]);
+    m0 = __reduce_max_sync(0xffffffffu, m0);
+    unsigned pi = 0xffffffffu;
+#pragma unroll
+    for (int i = NS - 1; i >= 0; --i)
+      if (khi[i] == m1 && klo[i] == m0 && lane + 32 * i < kx && !((gone >> i) & 1u)) pi = (unsigned)(lane + 32 * i);
+    pi = __reduce_min_sync(0xffffffffu, pi);
+    const double piv = __hiloint2double((int)m1, (int)m0);
+    if (!(piv > drop_tol) || pi >= (unsigned)kx) {    // the same decision in every warp
+      if (lane == 0) grank[0] = j;
+      break;
+    }
+    const int p = (int)pi;
+    if (scalar) {
+      // 1/piv to this CTA's rows
+      const double rp = rcp_full(piv);
+      if (lane == 0)
+        push_pair(&rbuf[par][32 * NS], &rbar[par], c, (unsigned)__double2loint(rp), (unsigned)__double2hiint(rp));
+    } else {
+      double rs = 0.0;
+#pragma unroll
+      for (int i = 0; i < NS; ++i)
+        if (i == (p >> 5)) rs = S[i];
+      rs = __shfl_sync(0xffffffffu, rs, p & 31);
+      if (lane < kXC)
+        push_pair(&rbuf[par][a], &rbar[par], lane, (unsigned)__double2loint(rs), (unsigned)__double2hiint(rs));
+      if (lane == 0) Lmine[wid * kx + j] = rs;
+      if (a == p) {                                   // this row is the pivot row
+        if (lane == 0) { gperm[j] = p; gpiv[j] = piv; }
+        break;
+      }
+      expired = !bar_wait(&rbar[par], ph);
+      if (__any_sync(0xffffffffu, expired)) { expired = true; break; }
+      const double f = -rs * (solo ? rcp_full(piv) : rbuf[par][32 * NS]);
+      if ((p & 31) == lane) gone |= 1u << (p >> 5);
+#pragma unroll
+      for (int i = 0; i < NS; ++i) {
+        const int b = lane + 32 * i;
+        const double rb = (b < kx && !((gone >> i) & 1u)) ? rbuf[par][b] : 0.0;
+        S[i] = fma(f, rb, S[i]);
+      }
+    }
+    if (scalar && (p & 31) == lane) gone |= 1u << (p >> 5);
+    if (p % kXC == c) --mine;
+  }
+  if (expired && lane == 0) grank[1] = 1;
+  cl.sync();                                          // pivots and rank complete; no more sends
+  const int rx = __ldcg(grank + 1) ? 0 : __ldcg(grank);
   for (int i = tid; i < kx; i += kXThreads) done[i] = 0;
   __syncthreads();
-  int rx = kx;
-  for (int j = 0; j < kx; ++j) {
-    const int par = j & 1;
-    if (wid == 0) {                                   // this CTA's candidate
-      unsigned long long best = 0ull;
-      int bi = kx;
-      for (int la = lane; la < nr; la += 32) {
-        const int a = c + kXC * la;
-        if (a < kx && !done[a]) {
-          const unsigned long long key = pivot_key(Srow[la * kx + a]);
-          if (key > best || (key == best && a < bi)) { best = key; bi = a; }
-        }
-      }
-      warp_argmax(best, bi);
-      if (lane == 0) { candk[par] = best; candi[par] = bi; }
-    }
-    cl.sync();
-    if (wid == 0) {                                   // the cluster's pivot
-      unsigned long long best = 0ull;
-      int bi = kx;
-      if (lane < kXC) {
-        best = *cl.map_shared_rank(&candk[par], lane);
-        bi = *cl.map_shared_rank(&candi[par], lane);
-      }
-      warp_argmax(best, bi);
-      if (lane == 0) {
-        const double piv = __longlong_as_double((long long)best);
-        s_go = piv > drop_tol && bi < kx;
-        s_p = bi;
-        s_piv = piv;
-      }
-    }
-    __syncthreads();
-    if (!s_go) { rx = j; break; }
-    const int p = s_p;
-    if (wid == 0) {                                   // 1/sqrt(piv), while the others stage row p
-      if (lane == 0) {
-        const double rl = rsqrt_nr(s_piv);
-        s_rl = rl;
-        perm[j] = p;
-        pos[p] = j;
-        rls[j] = rl;
-      }
-    } else {
-      const double* prow = cl.map_shared_rank(Srow, p % kXC) + (size_t)(p / kXC) * kx;
-      for (int b = tid - 32; b < kx; b += kXThreads - 32) lrow[b] = (done[b] || b == p) ? 0.0 : prow[b];
-    }
-    __syncthreads();
-    const double rl = s_rl;
-    for (int b = tid; b < kx; b += kXThreads) lrow[b] *= rl;   // column j of L (0 at eliminated indices)
-    __syncthreads();
-    // rank-1 update of this CTA's remaining rows (full rows: S stays exactly symmetric)
-    for (int la = wid; la < nr; la += nwarps) {
-      const int a = c + kXC * la;
-      if (a >= kx) continue;                          // warp-uniform
-      if (a == p) {
-        if (lane == 0) Lmine[la * kx + j] = s_piv * rl;
-        continue;
-      }
-      if (done[a]) continue;
-      const double l = lrow[a];
-      if (lane == 0) Lmine[la * kx + j] = l;
-      double* Sa = Srow + la * kx;
-      for (int b = lane; b < kx; b += 32) Sa[b] = fma(-l, lrow[b], Sa[b]);
-    }
-    if (tid == 0) done[p] = 1;
-    __syncthreads();
+  for (int q = tid; q < rx; q += kXThreads) {
+    const int p = __ldcg(gperm + q);
+    perm[q] = p;
+    pos[p] = q;
+    done[p] = 1;
+    rls[q] = rsqrt_nr(__ldcg(gpiv + q));
   }
-  cl.sync();                                          // no distributed shared-memory access after this
+  __syncthreads();
   // pivot order: the chosen indices, then the remaining ones in index order (one warp,
   // ballot prefix counts)
   if (wid == 0) {
@@ -531,14 +617,12 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
     }
   }
   __syncthreads();
-  // this CTA's rows of the factor, in pivot order, into w.S (every CTA read its rows
-  // of S_X before the first cluster barrier)
-  for (int la = wid; la < nr; la += nwarps) {
-    const int a = c + kXC * la;
-    if (a >= kx) continue;
+  // this CTA's rows of the factor, in pivot order, into w.S (every CTA read its rows of S_X
+  // before the first cluster barrier)
+  if (has) {
     const int pa = pos[a];
     for (int q = lane; q < kx; q += 32)
-      w.S[pa * kx + q] = (q < rx && q <= pa) ? Lmine[la * kx + q] : 0.0;
+      w.S[pa * kx + q] = (q < rx && q <= pa) ? Lmine[wid * kx + q] * rls[q] : 0.0;
   }
   cl.sync();                                          // w.S complete and visible in the cluster
   const int rank = nq + rx;
@@ -654,46 +738,6 @@ __device__ __forceinline__ float start_value(int a, int j, unsigned salt) {
 }
 // Solves per eigenvector (each followed by orthonormalisation inside the clusters).
 constexpr int kInvIters = 3;
-// Exchange of one 8-byte value per row among the CTAs of a cluster without a cluster
-// barrier: a row's warp stores its value into the slot of that row in every CTA
-// (st.async, lane q to CTA q), and the store counts its bytes on that CTA's mbarrier; a CTA's
-// readers wait on their own mbarrier for the bytes of all rows of the step.  The
-// barrier.cluster form has to wait for the acknowledgement of the stores before it arrives:
-// a Householder step took 2.0 us with it, 0.6 us with this.
-__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void push_pair(const void* slot, const void* bar, int rank, unsigned lo, unsigned hi) {
-  unsigned a, m;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(slot)), "r"(rank));
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(m) : "r"(smem_u32(bar)), "r"(rank));
-  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(a), "r"(lo),
-               "r"(hi), "r"(m)
-               : "memory");
-}
-__device__ __forceinline__ void bar_init(unsigned long long* bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void bar_expect(unsigned long long* bar, unsigned bytes) {
-  asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
-}
-// Waits for the phase of the given parity; false after about a second (the callers then
-// leave their loops, and the solve reports the result as not finite).
-__device__ __forceinline__ bool bar_wait(unsigned long long* bar, unsigned parity) {
-  const long long t0 = clock64();
-  while (true) {
-    unsigned done;
-    asm volatile(
-        "{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-        "selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (clock64() - t0 > 2000000000LL) return false;
-  }
-}
-
 // Householder tridiagonalisation of sym(T), eigenvalues by multisection of the Sturm
 // count, and the clusters and shifts of the inverse iteration, on a cluster of kEC
 // CTAs (one per SM).  A step is a chain of dependent operations, so the kernel is built to
@@ -1809,6 +1853,14 @@ void trsm(const double* Ahat, const double* Mhat, int n, double sigma, int pass,
     default: trsm_ns<kRowsPerLane>(Ahat, Mhat, n, sigma, pass, w, s); break;
   }
 }
+// Pivoted Cholesky launch: a warp per row of the kx <= 32 NS new columns.
+template <int NS>
+void xfactor(int n, int nq, int kx, const DW& w, double drop_tol, cudaStream_t s) {
+  const int sm = (int)((size_t)(32 * NS / kXC) * kx * sizeof(double));
+  BMG_CUDA(cudaFuncSetAttribute(xfactor_cl_kernel<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+  xfactor_cl_kernel<NS><<<kXC, 32 * (32 * NS / kXC + 1), sm, s>>>(n, nq, kx, w, drop_tol);
+  check_launch("xfactor_cl_kernel");
+}
 // FP32 eigensolve launch: a warp per row, n <= 32 NS rows over the cluster.
 template <int NS>
 void eig32(int n, const DW& w, cudaStream_t s) {
@@ -1863,10 +1915,15 @@ void dense_eig(const double* Ahat, const double* Mhat, int n, double sigma, int 
   const int nt = (kx + 7) / 8;
   schur_kernel<<<dim3(nt, nt), 64, 0, s>>>(Mhat, n, nq, kx, w);
   check_launch("schur_kernel");
-  const size_t xfs = 2 * (size_t)((kx + kXC - 1) / kXC) * kx * sizeof(double);
-  BMG_CUDA(cudaFuncSetAttribute(xfactor_cl_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xfs));
-  xfactor_cl_kernel<<<kXC, kXThreads, xfs, s>>>(n, nq, kx, w, drop_tol);
-  check_launch("xfactor_cl_kernel");
+  switch ((kx + 31) / 32) {
+    case 1: xfactor<1>(n, nq, kx, w, drop_tol, s); break;
+    case 2: xfactor<2>(n, nq, kx, w, drop_tol, s); break;
+    case 3: xfactor<3>(n, nq, kx, w, drop_tol, s); break;
+    case 4: xfactor<4>(n, nq, kx, w, drop_tol, s); break;
+    case 5: xfactor<5>(n, nq, kx, w, drop_tol, s); break;
+    case 6: xfactor<6>(n, nq, kx, w, drop_tol, s); break;
+    default: xfactor<7>(n, nq, kx, w, drop_tol, s); break;
+  }
   // 2. reduced standard matrix
   trsm(Ahat, Mhat, n, sigma, 0, w, s);
   trsm(Ahat, Mhat, n, sigma, 1, w, s);
