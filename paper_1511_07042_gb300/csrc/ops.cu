@@ -539,59 +539,98 @@ __global__ void row_norms_kernel(const int* __restrict__ row_ptr, const T* __res
 }
 
 // ---- transfers ----------------------------------------------------------------
+// Both kernels: one thread per (row, 16-byte chunk); its row by one multiplication (a 64-bit
+// division takes as many instructions as the rest of the kernel).  The chain of index loads before the
+// gathers (row order, then parents; row order, row extent, then midpoints) is hidden by the
+// number of threads: warps that take rows in turn with the chain run ahead were slower
+// (655362 x 128 float64, restriction and added prolongation: 854 us).
+// What bounds the float64 form is the float64 unit (85 % busy): an addition and a
+// multiply-add a value of an added prolongation, six multiply-adds a value of a restriction.
+// half_of(v) = v / 2 exactly: a float64 product holds the float64 unit for 64 cycles a
+// warp, which is most of what these kernels compute, so the exponent is lowered instead.
+__device__ __forceinline__ float half_of(float v) { return 0.5f * v; }
+__device__ __forceinline__ double half_of(double v) {
+  const int hi = __double2hiint(v), e = hi & 0x7FF00000;
+  if (e < 0x00200000 || e == 0x7FF00000) return 0.5 * v;   // zero, subnormal result, Inf or NaN
+  return __hiloint2double(hi - 0x00100000, __double2loint(v));
+}
+
+// t / d and t % d for t < 2^31 and a divisor of the launch: t / d = (t mul) >> (31 + sh) with
+// mul = ceil(2^(31 + sh) / d), sh = ceil(log2 d) (Granlund & Montgomery 1994: exact for 31-bit t).
+struct RowDiv {
+  unsigned d, mul, sh;
+};
+__device__ __forceinline__ void row_of(const RowDiv& v, unsigned t, int& row, int& c) {
+  const unsigned q = (unsigned)(((unsigned long long)t * v.mul) >> (31 + v.sh));
+  row = (int)q;
+  c = (int)(t - q * v.d);
+}
+
 // Y[v] (+)= P Xc: parents (a, b) of fine vertex v; a == b: copy, else the mean.
 // order (optional): the fine rows in Morton order of their positions, so that the
 // parents gathered by neighbouring threads are near one another in space and found in
 // L2 (each row is computed alone: the result does not depend on the order).
-template <typename T>
+template <typename T, bool ADD>
 __global__ void prolong_kernel(const int* __restrict__ par, int nf, const T* __restrict__ Xc,
-                               T* __restrict__ Y, int nch, int add, const int* __restrict__ order) {
+                               T* __restrict__ Y, RowDiv div, const int* __restrict__ order) {
   constexpr int W = Chunk<T>::W;
-  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (size_t)nf * nch) return;
-  const int v = order ? order[t / nch] : (int)(t / nch), c = (int)(t % nch);
-  const int a = par[2 * v], b = par[2 * v + 1];
-  T r[W];
-  ldv(Xc, (size_t)a * nch + c, r);
-  if (a != b) {
-    T y[W];
-    ldv(Xc, (size_t)b * nch + c, y);
-#pragma unroll
-    for (int q = 0; q < W; ++q) r[q] = T(0.5) * (r[q] + y[q]);
-  }
-  if (add) {
+  int row, c;
+  row_of(div, blockIdx.x * blockDim.x + threadIdx.x, row, c);
+  if (row >= nf) return;
+  const int v = order ? order[row] : row, nch = (int)div.d;
+  const int2 p = reinterpret_cast<const int2*>(par)[v];
+  {
+    T r[W];
+    ldv(Xc, (size_t)p.x * nch + c, r);
     T o[W];
-    ldv(Y, (size_t)v * nch + c, o);
+    if (ADD) ldv(Y, (size_t)v * nch + c, o);
+    const bool mean = p.x != p.y;
+    if (__any_sync(__activemask(), mean)) {
+      // a copy in a warp of means: 1 x instead of 0.5 (x + y); 0.5 s is exact, so the
+      // multiply-add rounds once, as adding the mean does
+      T y[W];
+      ldv(Xc, (size_t)p.y * nch + c, y);
 #pragma unroll
-    for (int q = 0; q < W; ++q) r[q] = o[q] + r[q];
+      for (int q = 0; q < W; ++q) {
+        const T s = r[q] + y[q];
+        if (ADD) r[q] = fma(mean ? T(0.5) : T(1), mean ? s : r[q], o[q]);
+        else if (mean) r[q] = half_of(s);
+      }
+    } else if (ADD) {
+#pragma unroll
+      for (int q = 0; q < W; ++q) r[q] = o[q] + r[q];
+    }
+    stv(Y, (size_t)v * nch + c, r);
   }
-  stv(Y, (size_t)v * nch + c, r);
 }
 
 // Zc[i] = R[i] + sum over edges (i, j): R[mid(i,j)] / 2, in ascending fine index.
 // order (optional): the coarse rows in Morton order, as in prolong_kernel.
 template <typename T>
-__global__ void restrict_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
-                                const int* __restrict__ mid, int nc, const T* __restrict__ R,
-                                T* __restrict__ Z, const T* __restrict__ R2, T* __restrict__ Z2, int nch,
-                                const int* __restrict__ order) {
+__global__ void restrict_kernel(const int* __restrict__ row_ptr, const int* __restrict__ mid, int nc,
+                                const T* __restrict__ R, T* __restrict__ Z, const T* __restrict__ R2,
+                                T* __restrict__ Z2, RowDiv div, const int* __restrict__ order) {
   // blockIdx.y = 1: the second block pair of a two-block launch
   if (blockIdx.y == 1) { R = R2; Z = Z2; }
   constexpr int W = Chunk<T>::W;
-  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (size_t)nc * nch) return;
-  const int i = order ? order[t / nch] : (int)(t / nch), c = (int)(t % nch);
-  T acc[W];
-  ldv(R, (size_t)i * nch + c, acc);
-  for (int p = row_ptr[i]; p < row_ptr[i + 1]; ++p) {
-    const int m = mid[p];
-    if (m < 0) continue;
-    T r[W];
-    ldv(R, (size_t)m * nch + c, r);
+  int row, c;
+  row_of(div, blockIdx.x * blockDim.x + threadIdx.x, row, c);
+  if (row >= nc) return;
+  const int i = order ? order[row] : row, nch = (int)div.d;
+  const int b = row_ptr[i], e = row_ptr[i + 1];
+  {
+    T acc[W];
+    ldv(R, (size_t)i * nch + c, acc);
+    for (int p = b; p < e; ++p) {
+      const int m = mid[p];
+      if (m < 0) continue;
+      T r[W];
+      ldv(R, (size_t)m * nch + c, r);
 #pragma unroll
-    for (int q = 0; q < W; ++q) acc[q] = acc[q] + T(0.5) * r[q];
+      for (int q = 0; q < W; ++q) acc[q] = fma(T(0.5), r[q], acc[q]);   // 0.5 r is exact
+    }
+    stv(Z, (size_t)i * nch + c, acc);
   }
-  stv(Z, (size_t)i * nch + c, acc);
 }
 
 // ---- tall-skinny Gram  G = X^T Y  --------------------------------------------
@@ -1175,13 +1214,25 @@ void residual(const Mesh& m, const T* a, const T* mm, const T* X, const T* B, co
                    zero_shift);
 }
 
+// Division by the chunks of a row in the transfer kernels, over at most 2^31 - 1 threads.
+static RowDiv row_div(int rows, int nch) {
+  if ((long long)rows * nch > 0x7FFFFF00ll) fail(BMG_ERR_INVALID_ARG, "transfer of more than 2^31 chunks of 16 bytes");
+  RowDiv v{(unsigned)nch, 0u, 0u};
+  while ((1u << v.sh) < v.d) ++v.sh;
+  v.mul = (unsigned)(((1ull << (31 + v.sh)) + v.d - 1) / v.d);
+  return v;
+}
+
 template <typename T>
 void prolong(const Mesh& fine, const T* Xc, T* Y, int ld, bool add, cudaStream_t s) {
   const int nch = ld / Chunk<T>::W;
-  const size_t total = (size_t)fine.n * nch;
+  const RowDiv div = row_div(fine.n, nch);
+  const int grid = blocks_for((size_t)fine.n * nch, 256);
   prof_begin(KC_TRANSFER, s);
-  prolong_kernel<T><<<blocks_for(total, 256), 256, 0, s>>>(fine.parents.get(), fine.n, Xc, Y, nch, add ? 1 : 0,
-                                                            fine.row_order.get());
+  if (add)
+    prolong_kernel<T, true><<<grid, 256, 0, s>>>(fine.parents.get(), fine.n, Xc, Y, div, fine.row_order.get());
+  else
+    prolong_kernel<T, false><<<grid, 256, 0, s>>>(fine.parents.get(), fine.n, Xc, Y, div, fine.row_order.get());
   check_launch("prolong_kernel");
   const double nc = (fine.n + 6) / 4.0;  // vertices of the coarse level of a refined sphere
   prof_end(KC_TRANSFER, s, 8.0 * fine.n + tb<T>() * ld * (nc + fine.n * (add ? 2.0 : 1.0)), 1.0 * fine.n * ld);
@@ -1196,12 +1247,11 @@ void restrict_(const Mesh& coarse, const T* R, T* Zc, int ld, cudaStream_t s) {
 template <typename T>
 void restrict2_(const Mesh& coarse, const T* R, T* Zc, const T* R2, T* Zc2, int ld, cudaStream_t s) {
   const int nch = ld / Chunk<T>::W;
-  const size_t total = (size_t)coarse.n * nch;
   const int pairs = R2 ? 2 : 1;
+  const RowDiv div = row_div(coarse.n, nch);
   prof_begin(KC_TRANSFER, s);
-  restrict_kernel<T><<<dim3((unsigned)blocks_for(total, 256), pairs), 256, 0, s>>>(
-      coarse.row_ptr.get(), coarse.col.get(), coarse.mid.get(), coarse.n, R, Zc, R2, Zc2, nch,
-      coarse.row_order.get());
+  restrict_kernel<T><<<dim3((unsigned)blocks_for((size_t)coarse.n * nch, 256), pairs), 256, 0, s>>>(
+      coarse.row_ptr.get(), coarse.mid.get(), coarse.n, R, Zc, R2, Zc2, div, coarse.row_order.get());
   check_launch("restrict_kernel");
   const double nf = 4.0 * coarse.n - 6.0;
   prof_end(KC_TRANSFER, s, pairs * (8.0 * coarse.nnz + tb<T>() * ld * (nf + coarse.n)), pairs * 2.0 * nf * ld);
