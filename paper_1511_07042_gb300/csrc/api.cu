@@ -285,13 +285,17 @@ extern "C" bmg_status bmg_hierarchy(bmg_problem* p, int levels) {
     p->lev.resize(L + 1);
     for (int l = 1; l <= L; ++l) {
       p->lev[l].refinement = p->r0 + l - 1;
+      locality_order(p->meshOf(l), s);
       colour_level(p->meshOf(l), p->lev[l], s);
-      locality_order(p->meshOf(l), p->lev[l], s);
     }
     p->ops.clear();
     p->ops.resize(L + 1);
     p->norm1.assign(L + 1, 0.0);
-    DBuf<unsigned long long> um(1);
+    // the norms of every level and the products' error flag are read once, at the end
+    Workspace ws(sizeof(unsigned long long) * (L + 2), s);
+    unsigned long long* um = ws.get<unsigned long long>();
+    int* err = reinterpret_cast<int*>(um + L + 1);
+    BMG_CUDA(cudaMemsetAsync(um, 0, sizeof(unsigned long long) * (L + 2), s));
     for (int f = 2; f <= L; ++f) {
       p->ops[f].resize(f + 1);
       for (int j = f; j >= 1; --j) {
@@ -300,23 +304,22 @@ extern "C" bmg_status bmg_hierarchy(bmg_problem* p, int levels) {
         if (j < f) {
           o.a.alloc(mj.nnz);
           o.m.alloc(mj.nnz);
-          galerkin(p->meshOf(j + 1), mj, p->opA(f, j + 1), p->opM(f, j + 1), o.a.get(), o.m.get(), s);
+          galerkin(p->meshOf(j + 1), mj, p->opA(f, j + 1), p->opM(f, j + 1), o.a.get(), o.m.get(), err, s);
         }
         o.da.alloc(mj.n);
         o.dm.alloc(mj.n);
         extract_diag(mj, p->opA(f, j), p->opM(f, j), o.da.get(), o.dm.get(), s);
       }
       const Mesh& mf = p->meshOf(f);
-      BMG_CUDA(cudaMemsetAsync(um.get(), 0, sizeof(unsigned long long), s));
-      row_abs_max_kernel<<<grid_of(mf.n, 256), 256, 0, s>>>(mf.row_ptr.get(), mf.valA.get(), mf.n, um.get());
+      row_abs_max_kernel<<<grid_of(mf.n, 256), 256, 0, s>>>(mf.row_ptr.get(), mf.valA.get(), mf.n, um + f);
       check_launch("row_abs_max_kernel");
-      unsigned long long h = 0;
-      BMG_CUDA(cudaMemcpyAsync(&h, um.get(), sizeof(h), cudaMemcpyDeviceToHost, s));
-      BMG_CUDA(cudaStreamSynchronize(s));
-      double nrm;
-      std::memcpy(&nrm, &h, sizeof(nrm));
-      p->norm1[f] = nrm;
     }
+    std::vector<unsigned long long> h(L + 2);
+    BMG_CUDA(cudaMemcpyAsync(h.data(), um, sizeof(unsigned long long) * (L + 2), cudaMemcpyDeviceToHost, s));
+    BMG_CUDA(cudaStreamSynchronize(s));
+    ws.idle();
+    if ((int)(h[L + 1] & 0xffffffffull)) fail(BMG_ERR_MESH, "Galerkin product left the coarse pattern");
+    for (int f = 2; f <= L; ++f) std::memcpy(&p->norm1[f], &h[f], sizeof(double));
     p->L = L;
   });
 }

@@ -263,9 +263,9 @@ void colour_level(const Mesh& m, Level& lv, cudaStream_t s);
 void colour_mesh(const Mesh& m, Colouring& cl, bool distance2, cudaStream_t s);
 // distance-2 colouring of the level (Kaczmarz), rows in Morton order; once
 void colour_level2(const Mesh& m, Level& lv, cudaStream_t s);
-void locality_order(Mesh& m, Level& lv, cudaStream_t s);
+void locality_order(Mesh& m, cudaStream_t s);   // before the level's colourings
 void galerkin(const Mesh& fine, const Mesh& coarse, const double* fa, const double* fm,
-              double* ca, double* cm, cudaStream_t s);
+              double* ca, double* cm, int* err, cudaStream_t s);
 void extract_diag(const Mesh& m, const double* a, const double* mm, double* da, double* dm,
                   cudaStream_t s);
 void fill_sh_constants(double* c17);

@@ -756,10 +756,10 @@ constexpr int kInvIters = 3;
 //   those rows, the only ones that still read, sent them after they had read step j's.
 // At n = 170 a step takes 0.6 us; with the matrix in shared memory, five CTA barriers and two
 // cluster barriers it took 2.5 us and the kernel 460 us.
-// Then every CTA brackets its share of the eigenvalues by multisection (a warp of 32
-// points per eigenvalue), and CTA 0 gathers them, forms the clusters and shifts of the
-// inverse iteration and writes the tridiagonal matrix.  Every thread of every CTA passes the
-// same number of cluster barriers.
+// Then every CTA brackets its share of the eigenvalues by multisection (8 points per
+// eigenvalue), and CTA 0 gathers them, forms the clusters and shifts of the inverse
+// iteration and writes the tridiagonal matrix.  Every thread of every CTA passes the same
+// number of cluster barriers.
 constexpr int kEC = 8;
 template <int NS>
 __global__ void __cluster_dims__(kEC, 1, 1) __launch_bounds__(32 * 32 * NS / kEC)
@@ -770,6 +770,7 @@ eig32_cl_kernel(int n, DW w) {
   constexpr int kThreads = 32 * nwarps;
   __shared__ __align__(16) float2 buf[2][32 * NS];    // p_g and A_g,j+1 of every row
   __shared__ __align__(8) unsigned long long bars[2];
+  __shared__ float xs[nwarps][32 * NS];               // x of each warp, for reads across lanes
   __shared__ float d[kMaxN], e[kMaxN], e2[kMaxN], vb[kMaxN], lam[kMaxN];
   __shared__ float slo[32], shi[32];
   const int c = (int)cl.block_rank();
@@ -806,14 +807,25 @@ eig32_cl_kernel(int n, DW w) {
   for (int j = 0; j + 2 < r && j <= g && g < r; ++j) {
     const int j1 = j + 1, par = j & 1;
     if (arms && lane == 0) bar_expect(&bars[par], 8u * (unsigned)(r - j));
-    float part = 0.f, a0s = 0.f, a1s = 0.f;
+    float a1s = 0.f;
 #pragma unroll
     for (int i = 0; i < NS; ++i) {
-      if (lane + 32 * i > j1) part = fmaf(x[i], x[i], part);
-      if (i == (j1 >> 5)) { a0s = x[i]; a1s = A[i]; }
+      xs[wid][lane + 32 * i] = x[i];
+      if (i == (j1 >> 5)) a1s = A[i];
     }
-    const float a0 = __shfl_sync(0xffffffffu, a0s, j1 & 31);
     const float a1 = __shfl_sync(0xffffffffu, a1s, j1 & 31);   // A_g,j+1
+    __syncwarp();
+    // the sums of this step group their terms in a fixed way (here lanes from j + 2 on), so
+    // that the tridiagonal matrix, and with it the signs of the eigenvectors, is the same
+    // whatever number of CTAs and warps shares the work
+    float part = 0.f;
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      const int b = j + 2 + lane + 32 * i;
+      const float y = b < 32 * NS ? xs[wid][b] : 0.f;
+      part = fmaf(y, y, part);
+    }
+    const float a0 = xs[wid][j1];
     const float xn2 = warp_sumf(part);
     float beta = a0, t = 0.f, scale = 0.f;
     if (xn2 > 0.f) {
@@ -857,17 +869,27 @@ eig32_cl_kernel(int n, DW w) {
       ok = false;
       break;
     }
-    float pw[NS], old[NS], pd = 0.f;
+    float pw[NS], old[NS], pd[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) pd[i] = 0.f;
 #pragma unroll
     for (int i = 0; i < NS; ++i) {
       const int b = lane + 32 * i;
       const float2 q = buf[par][b];
       pw[i] = (b >= j1 && b < r) ? q.x : 0.f;
       old[i] = q.y;
-      pd = fmaf(pw[i], v[i], pd);
+      pd[i] = __fmul_rn(pw[i], v[i]);
     }
     const float pg = buf[par][g].x, p1 = buf[par][j1].x;
-    const float kk = 0.5f * t * warp_sumf(pd);
+    // p.v: a tree over the rows of each residue mod 8 (row = lane + 32 i: the slots i, then
+    // the lanes), then the residues in order
+    float tsum = ((pd[0] + pd[4]) + (pd[2] + pd[6])) + ((pd[1] + pd[5]) + (pd[3] + pd[7]));
+    tsum += __shfl_xor_sync(0xffffffffu, tsum, 16);
+    tsum += __shfl_xor_sync(0xffffffffu, tsum, 8);
+    float kk = 0.f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) kk += __shfl_sync(0xffffffffu, tsum, q);
+    kk *= 0.5f * t;
     const float wg = fmaf(-kk, vg, pg), w1 = fmaf(-kk, 1.f, p1);
 #pragma unroll
     for (int i = 0; i < NS; ++i) {
@@ -916,38 +938,41 @@ eig32_cl_kernel(int n, DW w) {
   const float span = fmaxf(fmaxf(fabsf(lo), fabsf(hi)), 1e-30f);
   const float pivmin = 1e-30f * fmaxf(span * span, 1.f);
   // --- eigenvalues by multisection of the Sturm count, CTA c taking the eigenvalues
-  // [c qn, (c + 1) qn), a warp one eigenvalue: each lane counts the eigenvalues below one of
-  // 32 interior points of the interval, which splits it into 33 parts; 5 rounds shrink the
-  // Gershgorin interval by 33^5 = 3.9e7, to the FP32 resolution of the spectrum
-  // (eigenvalues near 0 need no more: the refinement takes them to FP64).  A round is a
-  // chain of r dependent divisions, so wide splits beat more rounds (8 rounds of 9 parts
-  // took 1.6 times as long).
+  // [c qn, (c + 1) qn): a group of 8 lanes brackets one eigenvalue; each lane counts
+  // the eigenvalues below one of 8 interior points of the group's interval, which
+  // splits it into 9 parts; 8 rounds shrink the Gershgorin interval by 9^8 = 4.3e7, to
+  // the FP32 resolution of the spectrum (eigenvalues near 0 need no more: the
+  // refinement takes them to FP64).
   const int qn = (r + kEC - 1) / kEC, i0 = c * qn, i1 = min(r, i0 + qn);
-  if (i0 + wid < i1) {                                  // warp-uniform
-    const int i = i0 + wid;
-    const float frac = (float)(lane + 1) * (1.0f / 33.0f);
-    float a = lo - 1e-6f * span, b = hi + 1e-6f * span;
-    for (int round = 0; round < 5; ++round) {
-      const float wd = b - a;
-      const float xx = fmaf(wd, frac, a);
-      int cnt = 0;
-      float q = d[0] - xx;
-      if (fabsf(q) < pivmin) q = -pivmin;
-      cnt += q < 0.f;
-      for (int jj = 1; jj < r; ++jj) {
-        q = (d[jj] - xx) - __fdividef(e2[jj - 1], q);
+  {
+    const int grp = tid >> 3, sl = tid & 7;
+    const int gsh = lane & 24;
+    const float frac = (float)(sl + 1) * (1.0f / 9.0f);
+    if (i0 + 4 * wid < i1) {                            // warp-uniform
+      const int i = min(i0 + grp, i1 - 1);
+      float a = lo - 1e-6f * span, b = hi + 1e-6f * span;
+      for (int round = 0; round < 8; ++round) {
+        const float wd = b - a;
+        const float xx = fmaf(wd, frac, a);
+        int cnt = 0;
+        float q = d[0] - xx;
         if (fabsf(q) < pivmin) q = -pivmin;
         cnt += q < 0.f;
+        for (int jj = 1; jj < r; ++jj) {
+          q = (d[jj] - xx) - __fdividef(e2[jj - 1], q);
+          if (fabsf(q) < pivmin) q = -pivmin;
+          cnt += q < 0.f;
+        }
+        // counts grow with x: the first point with more than i eigenvalues below it
+        const unsigned m = (__ballot_sync(0xffffffffu, cnt > i) >> gsh) & 0xffu;
+        const int first = m ? __ffs(m) - 1 : 8;
+        const float na = (first == 0) ? a : fmaf(wd, (float)first * (1.0f / 9.0f), a);
+        const float nb = (first == 8) ? b : fmaf(wd, (float)(first + 1) * (1.0f / 9.0f), a);
+        a = na;
+        b = nb;
       }
-      // counts grow with x: the first point with more than i eigenvalues below it
-      const unsigned m = __ballot_sync(0xffffffffu, cnt > i);
-      const int first = m ? __ffs(m) - 1 : 32;
-      const float na = (first == 0) ? a : fmaf(wd, (float)first * (1.0f / 33.0f), a);
-      const float nb = (first == 32) ? b : fmaf(wd, (float)(first + 1) * (1.0f / 33.0f), a);
-      a = na;
-      b = nb;
+      if (sl == 0 && i0 + grp < i1) lam[i] = 0.5f * (a + b);
     }
-    if (lane == 0) lam[i] = 0.5f * (a + b);
   }
   cl.sync();                                            // every CTA's eigenvalues bracketed
   if (c == 0)

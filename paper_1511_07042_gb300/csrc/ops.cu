@@ -485,7 +485,10 @@ kaczmarz_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col, co
   const int e = live ? row_ptr[row + 1] : 0;
   gather_row<T, LPR, CPL>(col, va, vm, X, b, e - b, nch, sl, st, aa, mm);
   if (!live) return;
-  const T n_a = na[row], n_am = nam[row], n_m = nm[row];
+  // ||k_r||^2 = na - 2 s nam + s^2 nm as nested multiply-adds, and the quotient from its
+  // reciprocal with one correction (a float64 division takes about eight float64 operations,
+  // which are what bounds the kernel: 29 -> 24 a value)
+  const T n_a = na[row], n_am2 = T(-2) * nam[row], n_m = nm[row];
   T coef[CPL][W], sv[CPL][W];
 #pragma unroll
   for (int u = 0; u < CPL; ++u) {
@@ -501,8 +504,9 @@ kaczmarz_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col, co
 #pragma unroll
     for (int q = 0; q < W; ++q) {
       const T res = bb[q] - (aa[u][q] - sv[u][q] * mm[u][q]);
-      const T nrm = n_a - T(2) * sv[u][q] * n_am + sv[u][q] * sv[u][q] * n_m;
-      coef[u][q] = nrm > T(0) ? omega * res / nrm : T(0);
+      const T nrm = fma(sv[u][q], fma(sv[u][q], n_m, n_am2), n_a);
+      const T num = omega * res, y = recip(nrm), f = num * y;
+      coef[u][q] = nrm > T(0) ? fma(fma(-nrm, f, num), y, f) : T(0);
     }
   }
   for (int p = b; p < e; ++p) {
