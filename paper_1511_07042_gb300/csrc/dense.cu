@@ -68,13 +68,6 @@ __device__ __forceinline__ double rcp_nr(double x) {
   const double y = (double)(1.0f / (float)x);
   return y * fma(-x, y, 2.0);
 }
-// 1/x to float64 accuracy for x in the FP32 normal range: FP32 seed and one step of third
-// order, y (1 + e + e^2) with e = 1 - x y.
-__device__ __forceinline__ double rcp_full(double x) {
-  const double y = (double)(1.0f / (float)x);
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
 __device__ __forceinline__ float warp_sumf(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -454,14 +447,15 @@ __device__ __forceinline__ bool bar_wait(unsigned long long* bar, unsigned parit
 // the pivots' reciprocals.  Pivoting is logical: an eliminated index keeps its row and is
 // only marked, and the pivot order is assembled at the end.  A step is two exchanges:
 //   every remaining row sends its diagonal to all CTAs; every warp takes the same pivot p
-//   (largest key, then smallest index);
-//   every remaining row sends its element r_a of column p, while the extra warp of each CTA
-//   forms 1/piv; then row a subtracts (r_a / piv) r_b.
-// The unscaled r_a are kept and scaled by 1/sqrt(piv) at the end.  The buffers alternate with
-// the parity of the step, as in the tridiagonalisation below: a row sends in step j + 2 only
-// after all rows that remain in step j + 1 have sent there, and these, the only ones that
-// still read step j's values, had read them before.
-// At k = 128 a step took 2.3 us with the pivot row fetched between CTA and cluster barriers.
+//   (largest key; among equal ones the smallest index, or with nq = 0 the first place of a
+//   factorisation that swaps pivots into place, whose order the results are known by);
+//   the extra warp of each CTA forms 1/sqrt(piv) for its rows, every remaining row sends its
+//   entry l_a of the factor's column, and row a subtracts l_a l_b.
+// The buffers alternate with the parity of the step, as in the tridiagonalisation below: a
+// row sends in step j + 2 only after all rows that remain in step j + 1 have sent there, and
+// these, the only ones that still read step j's values, had read them before.
+// With the pivot row fetched from its owner between CTA and cluster barriers a step took
+// 2.3 us at k = 128; a one-CTA factorisation of a 170 x 170 matrix 4.1 us.
 constexpr int kXC = 8;
 template <int NS>
 __global__ void __cluster_dims__(kXC, 1, 1) __launch_bounds__(32 * (32 * NS / kXC + 1))
@@ -471,9 +465,9 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
   constexpr int nrow = 32 * NS / kXC;                 // rows of a CTA, one warp each
   constexpr int nwarps = nrow + 1, kXThreads = 32 * nwarps;
   extern __shared__ double xsm[];
-  double* Lmine = xsm;                                // nrow x kx: r_a of each step of this CTA's rows
-  __shared__ __align__(16) double kbuf[2][32 * NS], rbuf[2][32 * NS + 1];   // rbuf's last: 1/piv
-  __shared__ __align__(8) unsigned long long kbar[2], rbar[2];
+  double* Lmine = xsm;                                // nrow x kx: this CTA's rows of the factor, by step
+  __shared__ __align__(16) double kbuf[2][32 * NS], rbuf[2][32 * NS], sbuf[2];   // diagonals, l_a, 1/sqrt(piv)
+  __shared__ __align__(8) unsigned long long kbar[2], rbar[2], sbar[2];
   __shared__ double rls[kMaxN];
   __shared__ int perm[kMaxN], pos[kMaxN];
   __shared__ unsigned char done[kMaxN];
@@ -483,10 +477,10 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
     if (c == 0 && tid == 0) *w.rank = 0;
     return;
   }
-  // pivot order and values through global memory: gperm[j], gpiv[j], then the rank
+  // pivot order and reciprocal roots through global memory, then the rank
   int* gperm = w.srt;
   int* grank = w.cl;                                  // [0] rank, [1] a wait expired
-  double* gpiv = w.lam;
+  double* grl = w.lam;
   const bool scalar = wid == nrow;
   const int a = scalar ? kx : c + kXC * wid;          // this warp's row
   const bool has = a < kx;
@@ -498,12 +492,15 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
   }
   for (int q = tid; q < nrow * kx; q += kXThreads) Lmine[q] = 0.0;
   if (tid == 0) {
-    for (int q = 0; q < 2; ++q) { bar_init(&kbar[q]); bar_init(&rbar[q]); }
+    for (int q = 0; q < 2; ++q) { bar_init(&kbar[q]); bar_init(&rbar[q]); bar_init(&sbar[q]); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     if (c == 0) { grank[0] = kx; grank[1] = 0; }
   }
   cl.sync();
   unsigned gone = 0u;                                 // eliminated columns of this lane, a bit per slot
+  int place[NS];                                      // places of the lane's columns (nq = 0), else their indices
+#pragma unroll
+  for (int i = 0; i < NS; ++i) place[i] = lane + 32 * i;
   // Rows of this CTA still to eliminate.  The extra warp works while there are two: one of
   // them then remains, whose next values wait for the extra warp's, so that no buffer is
   // written again before the extra warp has read it.  The last row does its work itself.
@@ -515,7 +512,8 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
     const unsigned ph = (unsigned)(j >> 1) & 1u;
     if ((scalar || solo) && lane == 0) {
       bar_expect(&kbar[par], 8u * (unsigned)(kx - j));
-      bar_expect(&rbar[par], 8u * (unsigned)(kx - j) + (solo ? 0u : 8u));
+      bar_expect(&rbar[par], 8u * (unsigned)(kx - j));
+      if (!solo) bar_expect(&sbar[par], 8u);
     }
     if (!scalar) {
       double ds = 0.0;
@@ -544,44 +542,57 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
     for (int i = 0; i < NS; ++i)
       if (khi[i] == m1) m0 = max(m0, klo[i]);
     m0 = __reduce_max_sync(0xffffffffu, m0);
-    unsigned pi = 0xffffffffu;
+    unsigned pi = 0xffffffffu;                        // place << 16 | index
 #pragma unroll
-    for (int i = NS - 1; i >= 0; --i)
-      if (khi[i] == m1 && klo[i] == m0 && lane + 32 * i < kx && !((gone >> i) & 1u)) pi = (unsigned)(lane + 32 * i);
+    for (int i = 0; i < NS; ++i)
+      if (khi[i] == m1 && klo[i] == m0 && lane + 32 * i < kx && !((gone >> i) & 1u))
+        pi = min(pi, ((unsigned)place[i] << 16) | (unsigned)(lane + 32 * i));
     pi = __reduce_min_sync(0xffffffffu, pi);
     const double piv = __hiloint2double((int)m1, (int)m0);
-    if (!(piv > drop_tol) || pi >= (unsigned)kx) {    // the same decision in every warp
+    if (!(piv > drop_tol) || pi == 0xffffffffu) {     // the same decision in every warp
       if (lane == 0) grank[0] = j;
       break;
     }
-    const int p = (int)pi;
+    const int p = (int)(pi & 0xffffu);
+    if (nq == 0) {                                    // the column in place j moves to the pivot's
+#pragma unroll
+      for (int i = 0; i < NS; ++i)
+        if (place[i] == j) place[i] = (int)(pi >> 16);
+    }
     if (scalar) {
-      // 1/piv to this CTA's rows
-      const double rp = rcp_full(piv);
+      const double rl = rsqrt_nr(piv);
       if (lane == 0)
-        push_pair(&rbuf[par][32 * NS], &rbar[par], c, (unsigned)__double2loint(rp), (unsigned)__double2hiint(rp));
+        push_pair(&sbuf[par], &sbar[par], c, (unsigned)__double2loint(rl), (unsigned)__double2hiint(rl));
     } else {
       double rs = 0.0;
 #pragma unroll
       for (int i = 0; i < NS; ++i)
         if (i == (p >> 5)) rs = S[i];
       rs = __shfl_sync(0xffffffffu, rs, p & 31);
+      double rl;
+      if (solo) {
+        rl = rsqrt_nr(piv);
+      } else {
+        expired = !bar_wait(&sbar[par], ph);
+        if (__any_sync(0xffffffffu, expired)) { expired = true; break; }
+        rl = sbuf[par];
+      }
+      const double l = (a == p ? piv : rs) * rl;
       if (lane < kXC)
-        push_pair(&rbuf[par][a], &rbar[par], lane, (unsigned)__double2loint(rs), (unsigned)__double2hiint(rs));
-      if (lane == 0) Lmine[wid * kx + j] = rs;
+        push_pair(&rbuf[par][a], &rbar[par], lane, (unsigned)__double2loint(l), (unsigned)__double2hiint(l));
+      if (lane == 0) Lmine[wid * kx + j] = l;
       if (a == p) {                                   // this row is the pivot row
-        if (lane == 0) { gperm[j] = p; gpiv[j] = piv; }
+        if (lane == 0) { gperm[j] = p; grl[j] = rl; }
         break;
       }
       expired = !bar_wait(&rbar[par], ph);
       if (__any_sync(0xffffffffu, expired)) { expired = true; break; }
-      const double f = -rs * (solo ? rcp_full(piv) : rbuf[par][32 * NS]);
       if ((p & 31) == lane) gone |= 1u << (p >> 5);
 #pragma unroll
       for (int i = 0; i < NS; ++i) {
         const int b = lane + 32 * i;
-        const double rb = (b < kx && !((gone >> i) & 1u)) ? rbuf[par][b] : 0.0;
-        S[i] = fma(f, rb, S[i]);
+        const double lb = (b < kx && !((gone >> i) & 1u)) ? rbuf[par][b] : 0.0;
+        S[i] = fma(-l, lb, S[i]);
       }
     }
     if (scalar && (p & 31) == lane) gone |= 1u << (p >> 5);
@@ -597,7 +608,7 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
     perm[q] = p;
     pos[p] = q;
     done[p] = 1;
-    rls[q] = rsqrt_nr(__ldcg(gpiv + q));
+    rls[q] = __ldcg(grl + q);
   }
   __syncthreads();
   // pivot order: the chosen indices, then the remaining ones in index order (one warp,
@@ -622,7 +633,7 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
   if (has) {
     const int pa = pos[a];
     for (int q = lane; q < kx; q += 32)
-      w.S[pa * kx + q] = (q < rx && q <= pa) ? Lmine[wid * kx + q] * rls[q] : 0.0;
+      w.S[pa * kx + q] = (q < rx && q <= pa) ? Lmine[wid * kx + q] : 0.0;
   }
   cl.sync();                                          // w.S complete and visible in the cluster
   const int rank = nq + rx;
