@@ -575,11 +575,12 @@ __device__ __forceinline__ void row_of(const RowDiv& v, unsigned t, int& row, in
 // parents gathered by neighbouring threads are near one another in space and found in
 // L2 (each row is computed alone: the result does not depend on the order).
 template <typename T, bool ADD>
-__global__ void prolong_kernel(const int* __restrict__ par, int nf, const T* __restrict__ Xc,
+__global__ void prolong_kernel(const int* __restrict__ par, int row0, int nf, const T* __restrict__ Xc,
                                T* __restrict__ Y, RowDiv div, const int* __restrict__ order) {
   constexpr int W = Chunk<T>::W;
   int row, c;
   row_of(div, blockIdx.x * blockDim.x + threadIdx.x, row, c);
+  row += row0;
   if (row >= nf) return;
   const int v = order ? order[row] : row, nch = (int)div.d;
   const int2 p = reinterpret_cast<const int2*>(par)[v];
@@ -611,7 +612,7 @@ __global__ void prolong_kernel(const int* __restrict__ par, int nf, const T* __r
 // Zc[i] = R[i] + sum over edges (i, j): R[mid(i,j)] / 2, in ascending fine index.
 // order (optional): the coarse rows in Morton order, as in prolong_kernel.
 template <typename T>
-__global__ void restrict_kernel(const int* __restrict__ row_ptr, const int* __restrict__ mid, int nc,
+__global__ void restrict_kernel(const int* __restrict__ row_ptr, const int* __restrict__ mid, int row0, int nc,
                                 const T* __restrict__ R, T* __restrict__ Z, const T* __restrict__ R2,
                                 T* __restrict__ Z2, RowDiv div, const int* __restrict__ order) {
   // blockIdx.y = 1: the second block pair of a two-block launch
@@ -619,6 +620,7 @@ __global__ void restrict_kernel(const int* __restrict__ row_ptr, const int* __re
   constexpr int W = Chunk<T>::W;
   int row, c;
   row_of(div, blockIdx.x * blockDim.x + threadIdx.x, row, c);
+  row += row0;
   if (row >= nc) return;
   const int i = order ? order[row] : row, nch = (int)div.d;
   const int b = row_ptr[i], e = row_ptr[i + 1];
@@ -1219,8 +1221,9 @@ void residual(const Mesh& m, const T* a, const T* mm, const T* X, const T* B, co
 }
 
 // Division by the chunks of a row in the transfer kernels, over at most 2^31 - 1 threads.
-static RowDiv row_div(int rows, int nch) {
-  if ((long long)rows * nch > 0x7FFFFF00ll) fail(BMG_ERR_INVALID_ARG, "transfer of more than 2^31 chunks of 16 bytes");
+// rows of a launch whose threads, one per row and chunk, are numbered below 2^31
+static int rows_per_launch(int nch) { return 0x7FFFFF00 / nch; }
+static RowDiv row_div(int nch) {
   RowDiv v{(unsigned)nch, 0u, 0u};
   while ((1u << v.sh) < v.d) ++v.sh;
   v.mul = (unsigned)(((1ull << (31 + v.sh)) + v.d - 1) / v.d);
@@ -1230,14 +1233,17 @@ static RowDiv row_div(int rows, int nch) {
 template <typename T>
 void prolong(const Mesh& fine, const T* Xc, T* Y, int ld, bool add, cudaStream_t s) {
   const int nch = ld / Chunk<T>::W;
-  const RowDiv div = row_div(fine.n, nch);
-  const int grid = blocks_for((size_t)fine.n * nch, 256);
+  const RowDiv div = row_div(nch);
   prof_begin(KC_TRANSFER, s);
-  if (add)
-    prolong_kernel<T, true><<<grid, 256, 0, s>>>(fine.parents.get(), fine.n, Xc, Y, div, fine.row_order.get());
-  else
-    prolong_kernel<T, false><<<grid, 256, 0, s>>>(fine.parents.get(), fine.n, Xc, Y, div, fine.row_order.get());
-  check_launch("prolong_kernel");
+  for (int r0 = 0, r1; r0 < fine.n; r0 = r1) {
+    r1 = r0 + std::min(fine.n - r0, rows_per_launch(nch));
+    const int grid = blocks_for((size_t)(r1 - r0) * nch, 256);
+    if (add)
+      prolong_kernel<T, true><<<grid, 256, 0, s>>>(fine.parents.get(), r0, r1, Xc, Y, div, fine.row_order.get());
+    else
+      prolong_kernel<T, false><<<grid, 256, 0, s>>>(fine.parents.get(), r0, r1, Xc, Y, div, fine.row_order.get());
+    check_launch("prolong_kernel");
+  }
   const double nc = (fine.n + 6) / 4.0;  // vertices of the coarse level of a refined sphere
   prof_end(KC_TRANSFER, s, 8.0 * fine.n + tb<T>() * ld * (nc + fine.n * (add ? 2.0 : 1.0)), 1.0 * fine.n * ld);
 }
@@ -1252,11 +1258,14 @@ template <typename T>
 void restrict2_(const Mesh& coarse, const T* R, T* Zc, const T* R2, T* Zc2, int ld, cudaStream_t s) {
   const int nch = ld / Chunk<T>::W;
   const int pairs = R2 ? 2 : 1;
-  const RowDiv div = row_div(coarse.n, nch);
+  const RowDiv div = row_div(nch);
   prof_begin(KC_TRANSFER, s);
-  restrict_kernel<T><<<dim3((unsigned)blocks_for((size_t)coarse.n * nch, 256), pairs), 256, 0, s>>>(
-      coarse.row_ptr.get(), coarse.mid.get(), coarse.n, R, Zc, R2, Zc2, div, coarse.row_order.get());
-  check_launch("restrict_kernel");
+  for (int r0 = 0, r1; r0 < coarse.n; r0 = r1) {
+    r1 = r0 + std::min(coarse.n - r0, rows_per_launch(nch));
+    restrict_kernel<T><<<dim3((unsigned)blocks_for((size_t)(r1 - r0) * nch, 256), pairs), 256, 0, s>>>(
+        coarse.row_ptr.get(), coarse.mid.get(), r0, r1, R, Zc, R2, Zc2, div, coarse.row_order.get());
+    check_launch("restrict_kernel");
+  }
   const double nf = 4.0 * coarse.n - 6.0;
   prof_end(KC_TRANSFER, s, pairs * (8.0 * coarse.nnz + tb<T>() * ld * (nf + coarse.n)), pairs * 2.0 * nf * ld);
 }
