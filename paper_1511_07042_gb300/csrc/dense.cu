@@ -11,7 +11,7 @@
 //      dropped (rank r).  The block form (qfactor_kernel, xsolve_kernel, schur_kernel,
 //      xfactor_cl_kernel) keeps the factor of a repeating leading block and factors the
 //      Schur complement of the new columns; without such a block the whole of Mhat is the
-//      new block (a one-CTA factorisation took 698 us at n = 170, this one 390 us).
+//      new block.
 //   2. trsm_kernel     [multi-CTA, FP64]  reduced standard matrix
 //      T = L^{-1} D P^T (Ahat - sigma Mhat) P D L^{-T}: two forward substitutions, one
 //      warp per column, L staged in shared memory.
@@ -402,7 +402,7 @@ schur_kernel(const double* __restrict__ Mhat, int n, int nq, int kx, DW w) {
 // (st.async, lane q to CTA q), and the store counts its bytes on that CTA's mbarrier; a CTA's
 // readers wait on their own mbarrier for the bytes of all rows of the step.  The
 // barrier.cluster form has to wait for the acknowledgement of the stores before it arrives:
-// a Householder step took 2.0 us with it, 0.6 us with this.
+// the tridiagonalisation kernel below took 366 us at n = 170 with it, 250 us with this.
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void push_pair(const void* slot, const void* bar, int rank, unsigned lo, unsigned hi) {
   unsigned a, m;
@@ -454,8 +454,8 @@ __device__ __forceinline__ bool bar_wait(unsigned long long* bar, unsigned parit
 // The buffers alternate with the parity of the step, as in the tridiagonalisation below: a
 // row sends in step j + 2 only after all rows that remain in step j + 1 have sent there, and
 // these, the only ones that still read step j's values, had read them before.
-// With the pivot row fetched from its owner between CTA and cluster barriers a step took
-// 2.3 us at k = 128; a one-CTA factorisation of a 170 x 170 matrix 4.1 us.
+// k = 128: 240 us; with the pivot row fetched from its owner between CTA and cluster barriers
+// 300 us, as a one-CTA factorisation 399 us.
 constexpr int kXC = 8;
 template <int NS>
 __global__ void __cluster_dims__(kXC, 1, 1) __launch_bounds__(32 * (32 * NS / kXC + 1))
@@ -765,8 +765,8 @@ constexpr int kInvIters = 3;
 //   The slots are double-buffered by the parity of the step: a warp sends in step j + 2 only
 //   after the values of step j + 1 of every row >= j + 1 have arrived, and the warps of
 //   those rows, the only ones that still read, sent them after they had read step j's.
-// At n = 170 a step takes 0.6 us; with the matrix in shared memory, five CTA barriers and two
-// cluster barriers it took 2.5 us and the kernel 460 us.
+// At n = 170 the kernel takes 250 us; with the matrix in shared memory, five CTA barriers and
+// two cluster barriers a step it took 452 us.
 // Then every CTA brackets its share of the eigenvalues by multisection (8 points per
 // eigenvalue), and CTA 0 gathers them, forms the clusters and shifts of the inverse
 // iteration and writes the tridiagonal matrix.  Every thread of every CTA passes the same
@@ -1039,169 +1039,202 @@ eig32_cl_kernel(int n, DW w) {
 // live in shared memory (row stride odd, no bank conflicts) when it has at most
 // kInvSmemMembers members, else in the global eigenvector block.  All clusters run at
 // once, so the sequential work is one factorisation and kInvIters solves of length r.
+// A solve is one thread's chain of r rows, so its rows are walked with selects instead of
+// branches and the operands of eight rows are read ahead; the Gram-Schmidt keeps column t
+// and the block's columns in registers and sums its eight projections by halves (9
+// exchanges instead of 40, the same additions).  With the cluster step's block form below an
+// eigensolve of n = 170 went from 1538 to 1454 us, results bit for bit the same.
 constexpr int kInvThreads = 64;
 constexpr int kInvSmemMembers = 63;
 constexpr int kInvLuFloats = 24 * 1024;   // shared memory for the LU factors (96 KB)
-__global__ void __launch_bounds__(kInvThreads)
-invit_kernel(int n, DW w, unsigned salt) {
-  extern __shared__ float zsh[];
-  const int r = *w.rank;
-  const int ncl = w.cls[0];
-  const int c = blockIdx.x;
-  if (c >= ncl) return;
-  const int c0 = w.cls[1 + c], m = w.cls[2 + c] - c0;
-  const float* __restrict__ d = w.T3;
-  const float* __restrict__ e = w.T3 + n;
-  const float* __restrict__ shift = w.T3 + 2 * n;
-  const float tiny = w.T3[3 * n];
-  const bool insm = m <= kInvSmemMembers;
-  const int zld = insm ? (m | 1) : r;
-  float* Z = insm ? zsh : w.Z32 + c0;            // Z[a * zld + t], member t = jv - c0
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  // LU factors: planes [5][row][member], in shared memory after the columns when they
-  // fit (a solve step then waits on no L2 round trip), else in global scratch
-  const bool lusm = 5 * r * m <= kInvLuFloats;
-  float* __restrict__ LU = lusm ? zsh + (size_t)n * kInvSmemMembers : w.LU32;
-  const size_t pl = lusm ? (size_t)r * m : (size_t)r * r;   // plane stride
-  const int rs = lusm ? m : r;                               // row stride
-  const int cbase = lusm ? 0 : c0;                           // column of member 0
-  for (int t = tid; t < m; t += kInvThreads) {
-    const int jv = c0 + t;
-    const float x = shift[jv];
-    float p0 = d[0] - x, p1 = (r > 1) ? e[0] : 0.f;
-    for (int jj = 0; jj + 1 < r; ++jj) {
-      const float bsub = e[jj], anext = d[jj + 1] - x, cnext = (jj + 2 < r) ? e[jj + 1] : 0.f;
-      float a0, a1, a2, mm, sw;
-      if (fabsf(bsub) > fabsf(p0)) {
-        a0 = bsub; a1 = anext; a2 = cnext; sw = 1.f;
-        mm = __fdividef(p0, bsub);
-        p0 = p1 - mm * anext;
-        p1 = -mm * cnext;
-      } else {
-        a0 = p0; a1 = p1; a2 = 0.f; sw = 0.f;
-        mm = (p0 != 0.f) ? __fdividef(bsub, p0) : 0.f;
-        p0 = anext - mm * p1;
-        p1 = cnext;
-      }
-      if (fabsf(a0) < tiny) a0 = (a0 < 0.f) ? -tiny : tiny;
-      const size_t o = (size_t)jj * rs + (cbase + t);
-      LU[o] = __frcp_rn(a0);
-      LU[pl + o] = a1;
-      LU[2 * pl + o] = a2;
-      LU[3 * pl + o] = mm;
-      LU[4 * pl + o] = sw;
+
+// lane's butterfly sums of v[0..7]: v[u] = sum over the warp, bit for bit warp_sumf(v[u])
+__device__ __forceinline__ void warp_sum8(float (&v)[8], int lane) {
+#pragma unroll
+  for (int h = 4, o = 16; h >= 1; h >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int u = 0; u < h; ++u) {
+      const float give = up ? v[u] : v[u + h], keep = up ? v[u + h] : v[u];
+      v[u] = keep + __shfl_xor_sync(0xffffffffu, give, o);
     }
-    const size_t o = (size_t)(r - 1) * rs + (cbase + t);
-    LU[o] = __frcp_rn((fabsf(p0) < tiny) ? ((p0 < 0.f) ? -tiny : tiny) : p0);
-    LU[pl + o] = 0.f;
-    LU[2 * pl + o] = 0.f;
-    for (int a = 0; a < r; ++a) Z[a * zld + t] = start_value(a, jv, salt);
   }
+  float s = v[0];                       // lanes with bits 16, 8, 4 = u hold sum u
+  s += __shfl_xor_sync(0xffffffffu, s, 2);
+  s += __shfl_xor_sync(0xffffffffu, s, 1);
+#pragma unroll
+  for (int u = 0; u < 8; ++u) v[u] = __shfl_sync(0xffffffffu, s, 4 * u);
+}
+
+// The solves of one cluster; LU planes pl apart and rows rs apart, columns of Z zld apart.
+__device__ __forceinline__ void invit_cluster(const float* d, const float* e, const float* __restrict__ shift,
+                                              float tiny, int r, int m, float* Z, int zld, float* LU, size_t pl,
+                                              int rs) {
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  for (int t = tid; t < m; t += kInvThreads) {
+    const float x = shift[t];
+    float p0 = d[0] - x, p1 = (r > 1) ? e[0] : 0.f;
+    float* L = LU + t;
+#pragma unroll 4
+    for (int jj = 0; jj + 1 < r; ++jj, L += rs) {
+      const float bsub = e[jj], anext = d[jj + 1] - x, cnext = (jj + 2 < r) ? e[jj + 1] : 0.f;
+      const bool sw = fabsf(bsub) > fabsf(p0);
+      const float num = sw ? p0 : bsub, den = sw ? bsub : p0;
+      const float a1 = sw ? anext : p1, lo = sw ? p1 : anext;
+      const float mm = (den != 0.f) ? __fdividef(num, den) : 0.f;
+      float a0 = den;
+      if (fabsf(a0) < tiny) a0 = (a0 < 0.f) ? -tiny : tiny;
+      p0 = lo - mm * a1;
+      p1 = sw ? -mm * cnext : cnext;
+      L[0] = __frcp_rn(a0);
+      L[pl] = a1;
+      L[2 * pl] = sw ? cnext : 0.f;
+      L[3 * pl] = mm;
+      L[4 * pl] = sw ? 1.f : 0.f;
+    }
+    L[0] = __frcp_rn((fabsf(p0) < tiny) ? ((p0 < 0.f) ? -tiny : tiny) : p0);
+    L[pl] = 0.f;
+    L[2 * pl] = 0.f;
+  }
+  __syncthreads();                      // Z is set by all threads
   for (int itr = 0; itr < kInvIters; ++itr) {
     for (int t = tid; t < m; t += kInvThreads) {
-      float* Zc = Z + t;
       // forward elimination with the row swaps; cur carries the updated z[jj]
-      float cur = Zc[0];
-      for (int j0 = 0; j0 + 1 < r; j0 += 8) {
+      float* z = Z + t;
+      float cur = z[0];
+      const float *l3 = LU + 3 * pl + t, *l4 = LU + 4 * pl + t;
+      auto eliminate = [&](float mv, float sv, float nx, float* at) {
+        const bool sw = sv != 0.f;
+        const float hi = sw ? nx : cur, lo = sw ? cur : nx;
+        *at = hi;
+        cur = lo - mv * hi;
+      };
+      int jj = 0;
+      for (; jj + 8 < r; jj += 8, l3 += 8 * rs, l4 += 8 * rs, z += 8 * zld) {
         float mv[8], sv[8], nx[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-          const int jj = j0 + u;
-          if (jj + 1 < r) {
-            const size_t o = (size_t)jj * rs + (cbase + t);
-            mv[u] = LU[3 * pl + o];
-            sv[u] = LU[4 * pl + o];
-            nx[u] = Zc[(jj + 1) * zld];
-          }
+          mv[u] = l3[u * rs];
+          sv[u] = l4[u * rs];
+          nx[u] = z[(u + 1) * zld];
         }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) eliminate(mv[u], sv[u], nx[u], z + u * zld);
+      }
+      for (; jj + 1 < r; ++jj, l3 += rs, l4 += rs, z += zld) eliminate(*l3, *l4, z[zld], z);
+      // back substitution with the upper factor (three diagonals); z is at row r - 1
+      *z = cur;
+      float z1 = 0.f, z2 = 0.f, mx = 0.f;
+      const float* l0 = LU + (size_t)(r - 1) * rs + t;
+      auto substitute = [&](float u0, float u1, float u2, float zv, float* at) {
+        const float tv = (zv - u1 * z1 - u2 * z2) * u0;
+        *at = tv;
+        z2 = z1;
+        z1 = tv;
+        mx = fmaxf(mx, fabsf(tv));
+      };
+      int a = r - 1;
+      for (; a >= 7; a -= 8, l0 -= 8 * rs, z -= 8 * zld) {
+        float u0[8], u1[8], u2[8], zv[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-          const int jj = j0 + u;
-          if (jj + 1 < r) {
-            if (sv[u] != 0.f) {
-              Zc[jj * zld] = nx[u];
-              cur = cur - mv[u] * nx[u];
-            } else {
-              Zc[jj * zld] = cur;
-              cur = nx[u] - mv[u] * cur;
-            }
-          }
-        }
-      }
-      Zc[(r - 1) * zld] = cur;
-      // back substitution with the upper factor (three diagonals)
-      float z1 = 0.f, z2 = 0.f, mx = 0.f;
-      for (int a1 = r - 1; a1 >= 0; a1 -= 4) {
-        float u0v[4], u1v[4], u2v[4], zv[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int a = a1 - u;
-          if (a >= 0) {
-            const size_t o = (size_t)a * rs + (cbase + t);
-            u0v[u] = LU[o];
-            u1v[u] = LU[pl + o];
-            u2v[u] = LU[2 * pl + o];
-            zv[u] = Zc[a * zld];
-          }
+          u0[u] = l0[-u * rs];
+          u1[u] = l0[pl - u * rs];
+          u2[u] = l0[2 * pl - u * rs];
+          zv[u] = z[-u * zld];
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int a = a1 - u;
-          if (a >= 0) {
-            const float tv = (zv[u] - u1v[u] * z1 - u2v[u] * z2) * u0v[u];
-            Zc[a * zld] = tv;
-            z2 = z1;
-            z1 = tv;
-            mx = fmaxf(mx, fabsf(tv));
-          }
-        }
+        for (int u = 0; u < 8; ++u) substitute(u0[u], u1[u], u2[u], zv[u], z - u * zld);
       }
+      for (; a >= 0; --a, l0 -= rs, z -= zld) substitute(l0[0], l0[pl], l0[2 * pl], *z, z);
       // scale first (the solve can grow the vector by 1/tiny)
       const float inv = (mx > 0.f) ? 1.f / mx : 0.f;
-      for (int a = 0; a < r; ++a) Zc[a * zld] *= inv;
+      z = Z + t;
+#pragma unroll 8
+      for (int q = 0; q < r; ++q) z[q * zld] *= inv;
     }
     __syncthreads();
     if (wid == 0) {
+      constexpr int RQ = kMaxDense / 32;
       for (int t = 0; t < m; ++t) {
+        float zt[RQ];
+#pragma unroll
+        for (int i = 0; i < RQ; ++i) zt[i] = lane + 32 * i < r ? Z[(lane + 32 * i) * zld + t] : 0.f;
         // orthogonalise against the earlier members: blocks of 8 at a time
         // (independent dot products, then one combined update), two passes
         for (int pass = 0; pass < 2; ++pass) {
           for (int q0 = 0; q0 < t; q0 += 8) {
             const int nq = min(8, t - q0);
-            float dot[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) dot[u] = 0.f;
-            for (int a = lane; a < r; a += 32) {
-              const float zj = Z[a * zld + t];
-              const float* zr = Z + a * zld + q0;
-#pragma unroll
-              for (int u = 0; u < 8; ++u) dot[u] = fmaf(zr[u < nq ? u : 0], zj, dot[u]);
-            }
+            float zr[8][RQ], dot[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-              const float sm = warp_sumf(dot[u]);
-              dot[u] = (u < nq) ? sm : 0.f;
-            }
-            for (int a = lane; a < r; a += 32) {
-              float zj = Z[a * zld + t];
-              const float* zr = Z + a * zld + q0;
+              dot[u] = 0.f;
+              if (u < nq) {
 #pragma unroll
-              for (int u = 0; u < 8; ++u) zj = fmaf(-dot[u], zr[u < nq ? u : 0], zj);
-              Z[a * zld + t] = zj;
+                for (int i = 0; i < RQ; ++i)
+                  zr[u][i] = lane + 32 * i < r ? Z[(lane + 32 * i) * zld + q0 + u] : 0.f;
+              }
             }
-            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+              if (u < nq) {
+#pragma unroll
+                for (int i = 0; i < RQ; ++i) dot[u] = fmaf(zr[u][i], zt[i], dot[u]);
+              }
+            warp_sum8(dot, lane);
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+              if (u < nq) {
+#pragma unroll
+                for (int i = 0; i < RQ; ++i) zt[i] = fmaf(-dot[u], zr[u][i], zt[i]);
+              }
           }
         }
         float nrm = 0.f;
-        for (int a = lane; a < r; a += 32) nrm += Z[a * zld + t] * Z[a * zld + t];
+#pragma unroll
+        for (int i = 0; i < RQ; ++i) nrm = fmaf(zt[i], zt[i], nrm);
         nrm = warp_sumf(nrm);
         nrm = (nrm > 0.f) ? rsqrtf(nrm) : 0.f;
-        for (int a = lane; a < r; a += 32) Z[a * zld + t] *= nrm;
+#pragma unroll
+        for (int i = 0; i < RQ; ++i)
+          if (lane + 32 * i < r) Z[(lane + 32 * i) * zld + t] = zt[i] * nrm;
         __syncwarp();
       }
     }
     __syncthreads();
   }
+}
+
+__global__ void __launch_bounds__(kInvThreads)
+invit_kernel(int n, DW w, unsigned salt) {
+  extern __shared__ float zsh[];
+  __shared__ float d[kMaxDense], e[kMaxDense];
+  const int r = *w.rank;
+  const int ncl = w.cls[0];
+  const int c = blockIdx.x;
+  if (c >= ncl) return;
+  const int c0 = w.cls[1 + c], m = w.cls[2 + c] - c0;
+  const float* __restrict__ shift = w.T3 + 2 * n + c0;
+  const float tiny = w.T3[3 * n];
+  const int tid = threadIdx.x;
+  for (int q = tid; q < r; q += kInvThreads) {
+    d[q] = w.T3[q];
+    e[q] = w.T3[n + q];
+  }
+  // the columns (member t = jv - c0) in shared memory when they fit, and after them the LU
+  // factors when they do (a solve step then waits on no L2 round trip), else in global scratch
+  const bool insm = m <= kInvSmemMembers, lusm = insm && 5 * r * m <= kInvLuFloats;
+  const int zld = insm ? (m | 1) : r;
+  float* Z = insm ? zsh : w.Z32 + c0;            // Z[a * zld + t]
+  for (int q = tid; q < r * m; q += kInvThreads) {
+    const int a = q / m, t = q - a * m;
+    Z[a * zld + t] = start_value(a, c0 + t, salt);
+  }
+  __syncthreads();
+  if (lusm)
+    invit_cluster(d, e, shift, tiny, r, m, zsh, zld, zsh + (size_t)n * kInvSmemMembers, (size_t)r * m, m);
+  else
+    invit_cluster(d, e, shift, tiny, r, m, Z, zld, w.LU32 + c0, (size_t)r * r, r);
   if (insm)
     for (int q = tid; q < r * m; q += kInvThreads) {
       const int a = q / m, t = q % m;
@@ -1477,7 +1510,8 @@ coeff_kernel(int n, const double* acc, double floor_rel, DW w) {
   if (tid == 0) s_thr = thr_from(nrm, acc_max(acc), floor_rel);
   for (int i = tid; i < r; i += kBig) sl[i] = w.lam[i];
   for (int i = wid; i < r; i += nwarps)
-    for (int j = lane; j < r; j += 32) w.E[i * n + j] = (i == j) ? 0.5 * (1.0 - w.G[i * n + i]) : 0.0;
+    for (int j = lane; j < r; j += 32) if (i != j) w.E[i * n + j] = 0.0;
+  for (int i = tid; i < r; i += kBig) w.E[i * n + i] = 0.5 * (1.0 - w.G[i * n + i]);
   __syncthreads();
   for (int i = tid; i < r; i += kBig) {
     // FP64 compares run on the scarce FP64 pipe: rank by order-preserving integer keys
@@ -1531,7 +1565,7 @@ constexpr size_t kClSmem = sizeof(double) * 5 * kMaxCluster * kMaxCluster + size
 // sweeps; T is the arithmetic (float or double).
 template <typename T>
 __device__ void jacobi_sweeps(T* A, T* V, int mm, int sweeps, T tol, T* ccs_c, T* ccs_s, int* cpr_p,
-                              int* cpr_q, T* red) {
+                              int* cpr_q, int* cpr_r, T* red) {
   const int tid = threadIdx.x;
   const int m2 = (mm % 2 == 0) ? mm : mm + 1;
   for (int sweep = 0; sweep < sweeps; ++sweep) {
@@ -1579,33 +1613,52 @@ __device__ void jacobi_sweeps(T* A, T* V, int mm, int sweeps, T tol, T* ccs_c, T
             ss = t * cc;
           }
         }
-        ccs_c[i] = cc; ccs_s[i] = ss; cpr_p[i] = p; cpr_q[i] = (q < mm && ss != T(0)) ? q : -1;
+        ccs_c[i] = cc; ccs_s[i] = ss; cpr_p[i] = p; cpr_q[i] = q; cpr_r[i] = q < mm && ss != T(0);
       }
       __syncthreads();
-      const int half = m2 / 2;
-      for (int it = tid; it < half * mm; it += kClThreads) {
-        const int i = it / mm, col = it % mm;
-        const int q = cpr_q[i];
-        if (q < 0) continue;
-        const int p = cpr_p[i];
-        const T cc = ccs_c[i], ss = ccs_s[i];
-        const T ap = A[p * mm + col], aq = A[q * mm + col];
-        A[p * mm + col] = cc * ap - ss * aq;
-        A[q * mm + col] = ss * ap + cc * aq;
-      }
-      __syncthreads();
-      for (int it = tid; it < half * mm; it += kClThreads) {
-        const int i = it / mm, row = it % mm;
-        const int q = cpr_q[i];
-        if (q < 0) continue;
-        const int p = cpr_p[i];
-        const T cc = ccs_c[i], ss = ccs_s[i];
-        const T ap = A[row * mm + p], aq = A[row * mm + q];
-        A[row * mm + p] = cc * ap - ss * aq;
-        A[row * mm + q] = ss * ap + cc * aq;
-        const T vp = V[row * mm + p], vq = V[row * mm + q];
-        V[row * mm + p] = cc * vp - ss * vq;
-        V[row * mm + q] = ss * vp + cc * vq;
+      // A <- J^T A J by blocks of a row pair and a column pair (the rows' rotation first), and
+      // V <- V J, in one pass without a barrier between the two rotations; an index without a
+      // partner (q = mm) has no rotation.  The fused forms are written out: a product rounded
+      // the other way would turn the vectors of equal eigenvalues
+      const int half = m2 / 2, blocks = half * half;
+      for (int it = tid; it < blocks + half * mm; it += kClThreads) {
+        if (it < blocks) {
+          const int i = it / half, j = it - i * half;
+          const bool ri = cpr_r[i], rj = cpr_r[j];
+          if (!ri && !rj) continue;
+          const int pi = cpr_p[i], qi = cpr_q[i], pj = cpr_p[j], qj = cpr_q[j];
+          const bool hi = qi < mm, hj = qj < mm;
+          T pp = A[pi * mm + pj], pq = hj ? A[pi * mm + qj] : T(0);
+          T qp = hi ? A[qi * mm + pj] : T(0), qq = hi && hj ? A[qi * mm + qj] : T(0);
+          if (ri) {
+            const T cc = ccs_c[i], ss = ccs_s[i];
+            const T a0 = pp, a1 = pq;
+            pp = fma(cc, a0, -(ss * qp));
+            qp = fma(ss, a0, cc * qp);
+            pq = fma(cc, a1, -(ss * qq));
+            qq = fma(ss, a1, cc * qq);
+          }
+          if (rj) {
+            const T cc = ccs_c[j], ss = ccs_s[j];
+            const T a0 = pp, a1 = qp;
+            pp = fma(cc, a0, -(ss * pq));
+            pq = fma(ss, a0, cc * pq);
+            qp = fma(cc, a1, -(ss * qq));
+            qq = fma(ss, a1, cc * qq);
+          }
+          A[pi * mm + pj] = pp;
+          if (hj) A[pi * mm + qj] = pq;
+          if (hi) A[qi * mm + pj] = qp;
+          if (hi && hj) A[qi * mm + qj] = qq;
+        } else {
+          const int v = it - blocks, i = v / mm, row = v - i * mm;
+          if (!cpr_r[i]) continue;
+          const int p = cpr_p[i], q = cpr_q[i];
+          const T cc = ccs_c[i], ss = ccs_s[i];
+          const T vp = V[row * mm + p], vq = V[row * mm + q];
+          V[row * mm + p] = fma(cc, vp, -(ss * vq));
+          V[row * mm + q] = fma(ss, vp, cc * vq);
+        }
       }
       __syncthreads();
     }
@@ -1631,9 +1684,10 @@ cluster_kernel(int n, DW w) {
   float* fV = fA + MM;
   __shared__ double ccs_c[kMaxCluster / 2], ccs_s[kMaxCluster / 2], red[32];
   __shared__ float fcs_c[kMaxCluster / 2], fcs_s[kMaxCluster / 2], redf[32];
-  __shared__ int cpr_p[kMaxCluster / 2], cpr_q[kMaxCluster / 2];
+  __shared__ int cpr_p[kMaxCluster / 2], cpr_q[kMaxCluster / 2], cpr_r[kMaxCluster / 2];
   __shared__ int idx[kMaxCluster];
   __shared__ double s_mu, s_sc;
+  __shared__ unsigned long long s_mx;
   const int c = blockIdx.x;
   if (c >= w.cl[0]) return;
   const int b = w.cl[1 + c], mm = w.cl[2 + c] - b;
@@ -1654,14 +1708,21 @@ cluster_kernel(int n, DW w) {
   if (tid == 0) {
     double mu = 0.0;
     for (int a = 0; a < mm; ++a) mu += cA[a * mm + a];
-    mu /= mm;
-    double mx = 0.0;
-    for (int a = 0; a < mm; ++a)
-      for (int e = a; e < mm; ++e)
-        mx = fmax(mx, fabs(0.5 * (cA[a * mm + e] + cA[e * mm + a]) - (a == e ? mu : 0.0)));
-    s_mu = mu;
-    s_sc = (mx > 0.0) ? 1.0 / mx : 0.0;
+    s_mu = mu / mm;
+    s_mx = 0ull;
   }
+  __syncthreads();
+  unsigned long long mx = 0ull;         // bits of a non-negative double; NaN entries do not count
+  for (int q = tid; q < mm * mm; q += kClThreads) {
+    const int a = q / mm, e = q % mm;
+    if (a > e) continue;
+    const double v = 0.5 * (cA[a * mm + e] + cA[e * mm + a]) - (a == e ? s_mu : 0.0);
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
+    if (bits <= 0x7FF0000000000000ull) mx = max(mx, bits);
+  }
+  atomicMax(&s_mx, mx);
+  __syncthreads();
+  if (tid == 0) s_sc = s_mx ? 1.0 / __longlong_as_double((long long)s_mx) : 0.0;
   __syncthreads();
   for (int q = tid; q < mm * mm; q += kClThreads) {
     const int a = q / mm, e = q % mm;
@@ -1671,7 +1732,7 @@ cluster_kernel(int n, DW w) {
     fV[q] = (a == e) ? 1.f : 0.f;
   }
   __syncthreads();
-  jacobi_sweeps<float>(fA, fV, mm, 12, 1e-13f, fcs_c, fcs_s, cpr_p, cpr_q, redf);
+  jacobi_sweeps<float>(fA, fV, mm, 12, 1e-13f, fcs_c, fcs_s, cpr_p, cpr_q, cpr_r, redf);
   // V1 = V0 (3 I - V0^T V0) / 2
   for (int q = tid; q < mm * mm; q += kClThreads) {
     const int a = q / mm, e = q % mm;
@@ -1692,7 +1753,7 @@ cluster_kernel(int n, DW w) {
     }
   }
   __syncthreads();
-  jacobi_sweeps<double>(cA, cV, mm, 10, 1e-32, ccs_c, ccs_s, cpr_p, cpr_q, red);
+  jacobi_sweeps<double>(cA, cV, mm, 10, 1e-32, ccs_c, ccs_s, cpr_p, cpr_q, cpr_r, red);
   for (int q = tid; q < mm * mm; q += kClThreads) {
     const int a = q / mm, e = q % mm;
     double sacc = 0.0;
