@@ -357,12 +357,17 @@ spmm_am_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
   const int lane = threadIdx.x & 31, sl = lane % LPR;
   const int per_group = (blockDim.x >> 5) * RPW;
   const int ngroups = (n + per_group - 1) / per_group;
-  for (int g = blockIdx.x * groups, gc = 0; g < ngroups; ++g) {
-    if (gc == groups) { g += (gridDim.x - 1) * groups; gc = 0; if (g >= ngroups) break; }
-    ++gc;
-    const int w = g * per_group + (threadIdx.x >> 5) * RPW + lane / LPR;
-    const bool live = w < n;               // every lane takes part in the row's shuffles
-    const int row = live ? (order ? order[w] : w) : 0;
+  const int w0 = (threadIdx.x >> 5) * RPW + lane / LPR;
+  auto row_at = [&](int g) {             // of this part of the warp, -1: none
+    const int w = g * per_group + w0;
+    return g < ngroups && w < n ? (order ? __ldg(order + w) : w) : -1;
+  };
+  int nrow = row_at(blockIdx.x * groups);
+  for (int g = blockIdx.x * groups, gc = 0; g < ngroups;) {
+    const bool live = nrow >= 0;           // every lane takes part in the row's shuffles
+    const int row = live ? nrow : 0;
+    if (++gc == groups) { g += (gridDim.x - 1) * groups; gc = 0; }
+    nrow = row_at(++g);                    // ahead, see row_update_kernel
     T aa[CPL][W], mm[CPL][W];
 #pragma unroll
     for (int u = 0; u < CPL; ++u)
@@ -389,6 +394,14 @@ spmm_am_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
 //   MODE 2 (residual): out  = r
 // ZS: every shift is zero (the shifted problems of a solve at sigma = 0): r = b - A x
 // and d = dA_i, so M and its diagonal are not read and 1/d is formed once per row.
+// A row is a chain of loads (its number, its extent, its columns, the gathers, then B and the
+// diagonals), and a warp has one row in hand: the next row's number is read a row ahead, and
+// the diagonals and B beside the gathers.  Float64 blocks have no registers to hold both
+// through their gathers: with shifts they take the number ahead, without (fewer sums) B.
+// 655362 x 128 float32, two sweeps: 727 us -> 701 with B and the diagonals -> 690 with both;
+// 40962 x 64 float64 symmetric Gauss-Seidel with shifts 226 -> 225 -> 221; the float64 sweeps
+// of a 655362-vertex solve at zero shift take 41.3 to 42.2 ms with B ahead, 42.6 with the
+// number, 42.2 with neither.  The product above: 1190 -> 1176 us in float64.
 template <typename T, int LPR, int CPL, int MODE, bool ZS>
 __global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512, sizeof(T) == 8 ? 3 : 1)
 row_update_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
@@ -404,21 +417,37 @@ row_update_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
   const int lane = threadIdx.x & 31, sl = lane % LPR;
   const int per_group = (blockDim.x >> 5) * RPW;
   const int ngroups = (nrows + per_group - 1) / per_group;
-  for (int g = blockIdx.x * groups, gc = 0; g < ngroups; ++g) {
-    if (gc == groups) { g += (gridDim.x - 1) * groups; gc = 0; if (g >= ngroups) break; }
-    ++gc;
-    const int w = g * per_group + (threadIdx.x >> 5) * RPW + lane / LPR;
-    const bool live = w < nrows;           // every lane takes part in the row's shuffles
-    const int row = live ? (rows ? rows[w] : w) : 0;
+  constexpr bool kNext = sizeof(T) == 4 || !ZS;
+  const int w0 = (threadIdx.x >> 5) * RPW + lane / LPR;
+  auto row_at = [&](int g) {             // of this part of the warp, -1: none
+    const int w = g * per_group + w0;
+    return g < ngroups && w < nrows ? (rows ? __ldg(rows + w) : w) : -1;
+  };
+  int nrow = kNext ? row_at(blockIdx.x * groups) : 0;
+  for (int g = blockIdx.x * groups, gc = 0; g < ngroups;) {
+    const int at = kNext ? nrow : row_at(g);
+    const bool live = at >= 0;             // every lane takes part in the row's shuffles
+    const int row = live ? at : 0;
+    if (++gc == groups) { g += (gridDim.x - 1) * groups; gc = 0; }
+    ++g;
+    if (kNext) nrow = row_at(g);           // the next row's number, ahead
     T aa[CPL][W], mm[CPL][W];
 #pragma unroll
     for (int u = 0; u < CPL; ++u)
 #pragma unroll
       for (int q = 0; q < W; ++q) { aa[u][q] = T(0); mm[u][q] = T(0); }
     const int b = live ? row_ptr[row] : 0;
+    constexpr bool kAhead = sizeof(T) == 4 || ZS;
+    T bb[CPL][W];
+#pragma unroll
+    for (int u = 0; u < CPL; ++u) {
+#pragma unroll
+      for (int q = 0; q < W; ++q) bb[u][q] = T(0);
+      if (kAhead && B && live && sl + LPR * u < nch) ldv(B, (size_t)row * nch + sl + LPR * u, bb[u]);
+    }
+    const T dai = live ? __ldg(da + row) : T(0), dmi = (ZS || !live) ? T(0) : __ldg(dm + row);
     gather_row<T, LPR, CPL, !ZS, ZS ? 2 : 0>(col, va, vm, X, b, live ? row_ptr[row + 1] - b : 0, nch, sl, st, aa, mm);
     if (!live) continue;
-    const T dai = da[row], dmi = ZS ? T(0) : dm[row];
     const T rd0 = (ZS && MODE != 2) ? recip(dai) : T(0);
 #pragma unroll
     for (int u = 0; u < CPL; ++u) {
@@ -435,10 +464,9 @@ row_update_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
       for (int q = 0; q < W; ++q) r[q] = ZS ? -aa[u][q] : -(aa[u][q] - s[q] * mm[u][q]);
       const size_t idx = (size_t)row * nch + c;
       if (B) {
-        T bb[W];
-        ldv(B, idx, bb);
+        if (!kAhead) ldv(B, idx, bb[u]);
 #pragma unroll
-        for (int q = 0; q < W; ++q) r[q] += bb[q];
+        for (int q = 0; q < W; ++q) r[q] += bb[u][q];
       }
       if (MODE == 2) {
         stv_cs(Out, idx, r);
