@@ -84,7 +84,7 @@ __device__ __forceinline__ void stv(float* p, size_t i, const float (&v)[4]) {
 // small a), rows longer than kFixNnz, and values outside a band of exponents (zeros among
 // normal values excepted; Inf, NaN and subnormals fall outside) take the float64 loop.
 // Result and error do not depend on the lanes per row.
-// Measured, 655362 x 128: [AX | MX] 1924 -> 1194 us (NF = 2; 1418 and 1350 us with 1 and
+// Measured, 655362 x 128: [AX | MX] 1924 -> 1170 us (NF = 2; 1418 and 1350 us with 1 and
 // 3); now bound by the issue of about 55 integer instructions per product pair.
 constexpr int kFixNnz = 7;     // a vertex of a subdivided surface and its six neighbours
 constexpr int kFixSlack = 3;
@@ -344,8 +344,11 @@ __device__ __forceinline__ float recip(float d) { return __frcp_rn(d); }
 // stretches of the Morton row order (neighbour rows of X found in its L1), while all
 // SMs together stay within a window of the order that L2 holds (neighbours shared
 // across chunks found in L2).
+// float32: no count of resident blocks is asked for (0): asked for one, the compiler takes 60
+// to 72 registers a thread where 40 do, and two blocks fit instead of three (two float32
+// Jacobi sweeps at 655362 x 128: 690 us instead of 594).
 template <typename T, int LPR, int CPL>
-__global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512, sizeof(T) == 8 ? 3 : 1)
+__global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512, sizeof(T) == 8 ? 3 : 0)
 spmm_am_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
                const T* __restrict__ va, const T* __restrict__ vm,
                const T* __restrict__ X, int n, int nch, T* __restrict__ AX,
@@ -398,12 +401,13 @@ spmm_am_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
 // diagonals), and a warp has one row in hand: the next row's number is read a row ahead, and
 // the diagonals and B beside the gathers.  Float64 blocks have no registers to hold both
 // through their gathers: with shifts they take the number ahead, without (fewer sums) B.
-// 655362 x 128 float32, two sweeps: 727 us -> 701 with B and the diagonals -> 690 with both;
+// 655362 x 128 float32, two sweeps: 727 us -> 701 with B and the diagonals -> 690 with both
+// (-> 594 with the launch bound of the product above);
 // 40962 x 64 float64 symmetric Gauss-Seidel with shifts 226 -> 225 -> 221; the float64 sweeps
 // of a 655362-vertex solve at zero shift take 41.3 to 42.2 ms with B ahead, 42.6 with the
-// number, 42.2 with neither.  The product above: 1190 -> 1176 us in float64.
+// number, 42.2 with neither.  The product above: 1190 -> 1170 us in float64.
 template <typename T, int LPR, int CPL, int MODE, bool ZS>
-__global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512, sizeof(T) == 8 ? 3 : 1)
+__global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512, sizeof(T) == 8 ? 3 : 0)
 row_update_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
                   const T* __restrict__ va, const T* __restrict__ vm,
                   const T* __restrict__ da, const T* __restrict__ dm,
