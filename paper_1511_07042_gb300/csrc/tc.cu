@@ -39,18 +39,19 @@
 // columns).  Operand digits are written by 16 worker warps into shared memory in the
 // no-swizzle K-major core-matrix layout (8 rows x 16 bytes per core matrix), two
 // stages; one thread of a seventeenth warp issues tcgen05.mma (kind::f16, BF16 x BF16 ->
-// FP32, M = 128, N = 64 to 256) and commits to an mbarrier per stage, so that the digits of
+// FP32, M = 128, N = 128 to 256) and commits to an mbarrier per stage, so that the digits of
 // the next 32-row sub-chunk are formed while the tensor cores work on the current one;
 // three more warps gather the exponents ahead.  Every wait is bounded (about 2 s of clock);
 // on expiry the kernel raises *err, waits a bounded time more, frees its tensor memory and
 // returns.
 //
-// Measured, 655362 x 128, float64 (float32): Gram 1720 -> 1002 us (1200 -> 533),
-// expansion 2130 -> 1387 us (1270 -> 665).  The largest parts of it: one wide MMA for up to
-// four digit planes of B (Gram 1339 -> 1030 us), exponents by their own warps from L2 with
-// 16-byte loads (float32 Gram 901 -> 533 us), digits by float32 additions.  What bounds the
-// float64 forms now: the readback's and the digits' integer work at four warps a scheduler
-// (without the MMAs the Gram takes 950 us, without the readback 980 us).
+// Measured, 655362 x 128, float64 (float32): Gram 1720 -> 1030 us (1200 -> 578),
+// expansion 2130 -> 1430 us (1270 -> 705).  The largest parts of it: one wide MMA for several
+// digit planes of B, exponents by their own warps from L2 with 16-byte loads, digits by float32
+// additions.  One base and N for all MMAs of a group of accumulators (issue_mmas) adds a third
+// of zero products: 1002 and 1387 us (533 and 665) without it.  What bounds the float64 forms
+// now: the readback's and the digits' integer work at four warps a scheduler (before that
+// change, the Gram took 950 us without the MMAs and 980 us without the readback).
 #include <algorithm>
 #include <cstring>
 
@@ -77,7 +78,13 @@ constexpr int kAPlane = 128 * kKsub * 2;  // bytes per digit plane of the 128-ro
 constexpr int kBPlane = kNB * kKsub * 2;  // bytes per digit plane of the 64-row operand
 static_assert(kBPlane == (kNB / 8) * kKsub * 16, "planes of B one 8-row stride apart (issue_mmas)");
 
-__host__ __device__ constexpr int stage_bytes(int S) { return S * (kAPlane + kBPlane); }
+// Planes of the 64-row operand that one MMA multiplies (its N is kNB times that), and the zero
+// planes in front of them (issue_mmas); S digits: 8 of float64 blocks, 5 of float32 blocks.
+__host__ __device__ constexpr int mma_planes(int S) { return S == 8 ? 4 : 3; }
+__host__ __device__ constexpr int zero_planes(int S) { return mma_planes(S) - 1; }
+__host__ __device__ constexpr int stage_bytes(int S) { return S * kAPlane + (zero_planes(S) + S) * kBPlane; }
+// offset of the first digit plane of the 64-row operand in a stage
+__host__ __device__ constexpr int b_offset(int S) { return S * kAPlane + zero_planes(S) * kBPlane; }
 
 // byte offset of the 8-element K-group starting at (row, k0) (k0 % 8 == 0)
 __device__ __forceinline__ int cm_off(int row, int k0) {
@@ -276,29 +283,79 @@ template <> struct Digits<double> {
   }
 };
 
-// Issues the MMAs of one sub-chunk: every digit pair (s, t) with s + t <= T into the
-// accumulator of its diagonal (columns (s + t - 2) * kNB of the allocation).  The planes of
-// the B operand follow one another at the stride of its 8-row groups, and the diagonals of
-// s and consecutive t are consecutive accumulators, so one MMA of N = kNB m multiplies
-// plane s of A with m <= 4 planes of B: the A plane is read from shared memory once for
-// them, and 12 (float32: 7) wide MMAs take the place of 36 (15) of N = 64, which the reads
-// of their operands held to a third of the tensor rate.
-// first: the sub-chunk opens an accumulation window (plane 1 of A reaches every diagonal
-// and overwrites it).
+// The MMAs of one K-step of a sub-chunk: every digit pair (s, t) with s + t <= T into the
+// accumulator of its diagonal, the kNB columns from (s + t - 2) * kNB of the allocation.
+//
+// The planes of the B operand follow one another at the stride of its 8-row groups, and the
+// diagonals of s and consecutive t are consecutive accumulators, so that one MMA of
+// N = kNB m multiplies plane s of A with m planes of B: the A plane is read from shared
+// memory once for them (MMAs of N = 64 were held to a third of the tensor rate by the reads of
+// their operands).  tcgen05.mma are executed in the order of issue only where they have the
+// same accumulator and the same shape; others may overtake one another, and an accumulation
+// or the overwriting at the start of a window would be lost.  The accumulators are therefore
+// taken in fixed groups of mma_planes(S) diagonals, and every MMA that writes a group has the
+// group's base and N: where a group begins before the diagonal of (s, 1), the first planes
+// of B are the zero planes in front of plane 1, which add nothing.
+// 12 MMAs of N = 256 for float64 digits, 3 of N = 192 and 5 of 128 for float32 digits (655362
+// x 128: Gram 1030 us and 578 us; in groups of two 1099 and 613, of three float64 and four
+// float32 diagonals 1072 and 599).
+struct MmaOp {
+  int s, t, col, n;   // plane of A, first plane of B (below 1: a zero plane), columns
+};
+template <int S, int T>
+struct MmaPlan {
+  int count = 0;
+  MmaOp op[S * T] = {};
+  __host__ __device__ constexpr MmaPlan() {
+    constexpr int W = mma_planes(S);
+    for (int s = 1; s <= S; ++s)
+      for (int d = 0; d <= T - 2; d += W) {            // diagonals s + t - 2 = d .. d + m - 1
+        const int m = T - 1 - d < W ? T - 1 - d : W, t = d - s + 2;
+        if (t + m - 1 >= 1) op[count++] = {s, t, d * kNB, m * kNB};
+      }
+  }
+  // every pair once and nothing else but zero planes, the first MMA of each group covering it,
+  // and one base and N for all MMAs that share a column
+  constexpr bool sound() const {
+    int seen[S + 1][S + 1] = {};
+    for (int q = 0; q < count; ++q) {
+      const MmaOp& a = op[q];
+      if (a.t < 1 - zero_planes(S) || a.col + a.n > (T - 1) * kNB || a.n > 256) return false;
+      for (int v = 0; v < a.n / kNB; ++v) {
+        const int t = a.t + v;
+        if (t > S || a.s + t - 2 != a.col / kNB + v) return false;
+        if (t >= 1) ++seen[a.s][t];
+      }
+      for (int p = 0; p < q; ++p) {
+        const MmaOp& b = op[p];
+        if (a.col < b.col + b.n && b.col < a.col + a.n && (a.col != b.col || a.n != b.n)) return false;
+      }
+      bool opens = true;                               // the first writer of its columns is plane 1
+      for (int p = 0; p < q; ++p) opens = opens && op[p].col != a.col;
+      if (opens != (a.s == 1)) return false;
+    }
+    for (int s = 1; s <= S; ++s)
+      for (int t = 1; t <= S; ++t)
+        if (seen[s][t] != (s + t <= T ? 1 : 0)) return false;
+    return true;
+  }
+};
+static_assert(MmaPlan<Digits<double>::S, Digits<double>::T>().sound(), "MMAs of float64 digits");
+static_assert(MmaPlan<Digits<float>::S, Digits<float>::T>().sound(), "MMAs of float32 digits");
+
+// Issues the MMAs of one sub-chunk (sB: the first zero plane of B).  first: the sub-chunk opens
+// an accumulation window (plane 1 of A reaches every diagonal and overwrites it).
 template <int S, int T>
 __device__ __forceinline__ void issue_mmas(uint32_t tmem, uint32_t sA, uint32_t sB, bool first) {
+  constexpr MmaPlan<S, T> plan;
 #pragma unroll
   for (int ks = 0; ks < kKsub / 16; ++ks) {
 #pragma unroll
-    for (int s = 1; s <= S; ++s) {
-#pragma unroll
-      for (int t = 1; t <= T - s; t += 4) {
-        const int m = T - s - t + 1 < 4 ? T - s - t + 1 : 4;
-        const uint64_t ad = sdesc(sA + (s - 1) * kAPlane + ks * 256, 128, kKsub * 16);
-        const uint64_t bd = sdesc(sB + (t - 1) * kBPlane + ks * 256, 128, kKsub * 16);
-        mma_bf16(tmem + (uint32_t)((s + t - 2) * kNB), ad, bd, idesc_bf16(128, kNB * m),
-                 (first && s == 1 && ks == 0) ? 0u : 1u);
-      }
+    for (int q = 0; q < plan.count; ++q) {
+      const MmaOp op = plan.op[q];
+      const uint64_t ad = sdesc(sA + (op.s - 1) * kAPlane + ks * 256, 128, kKsub * 16);
+      const uint64_t bd = sdesc(sB + (op.t - 1 + zero_planes(S)) * kBPlane + ks * 256, 128, kKsub * 16);
+      mma_bf16(tmem + (uint32_t)op.col, ad, bd, idesc_bf16(128, op.n), (first && op.s == 1 && ks == 0) ? 0u : 1u);
     }
   }
 }
@@ -519,7 +576,7 @@ __device__ __forceinline__ bool mma_step(TcShared& sh, unsigned char* smem, uint
   if (lane == 0 && !sh.no_mma) {
     fence_after();
     const uint32_t sA = su32(stage_ptr<S>(smem, b));
-    issue_mmas<S, T>(tmem, sA, sA + S * kAPlane, sc == 0);
+    issue_mmas<S, T>(tmem, sA, sA + S * kAPlane, sc == 0);   // (the zero planes follow the planes of A)
     mma_commit(&sh.bar[b]);
   }
   __syncwarp();
@@ -751,7 +808,7 @@ gram_tc_kernel(const TI* __restrict__ X, const TI* __restrict__ Y, int n, int k,
       if (g >= 2) wait_sub(sh, g - 2);
       unsigned char* st = stage_ptr<S>(smem, b);
       if (has_x) Digits<TI>::store(vx, EA, st + cm_off(cx, kx * 8), kAPlane);
-      if (do_y) Digits<TI>::store(vy, EB, st + S * kAPlane + cm_off(cy, ky * 8), kBPlane);
+      if (do_y) Digits<TI>::store(vy, EB, st + b_offset(S) + cm_off(cy, ky * 8), kBPlane);
       if (sc == 0 && w > 0) {
         wait_sub(sh, g - 1);
         __syncwarp();
@@ -1057,7 +1114,7 @@ expand_tc_kernel(const TI* __restrict__ Z, const TI* __restrict__ X, const unsig
           if (tid + q * kWorkers < S * kBPlane / 16) yd[q] = __ldg(src + tid + q * kWorkers);
         if (g >= 2) wait_sub(sh, g - 2);
         unsigned char* st = stage_ptr<S>(smem, b);
-        uint4* dst = reinterpret_cast<uint4*>(st + S * kAPlane);
+        uint4* dst = reinterpret_cast<uint4*>(st + b_offset(S));
 #pragma unroll
         for (int q = 0; q < NC; ++q)
           if (tid + q * kWorkers < S * kBPlane / 16) dst[tid + q * kWorkers] = yd[q];
