@@ -403,6 +403,9 @@ schur_kernel(const double* __restrict__ Mhat, int n, int nq, int kx, DW w) {
 // readers wait on their own mbarrier for the bytes of all rows of the step.  The
 // barrier.cluster form has to wait for the acknowledgement of the stores before it arrives:
 // the tridiagonalisation kernel below took 366 us at n = 170 with it, 250 us with this.
+// An asynchronous store is complete only when its mbarrier says so (a cluster barrier does not
+// wait for it), and a CTA must not leave while one is on its way to it.  A value is therefore
+// sent only to CTAs in which some warp waits for all values of that step.
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void push_pair(const void* slot, const void* bar, int rank, unsigned lo, unsigned hi) {
   unsigned a, m;
@@ -453,7 +456,9 @@ __device__ __forceinline__ bool bar_wait(unsigned long long* bar, unsigned parit
 //   entry l_a of the factor's column, and row a subtracts l_a l_b.
 // The buffers alternate with the parity of the step, as in the tridiagonalisation below: a
 // row sends in step j + 2 only after all rows that remain in step j + 1 have sent there, and
-// these, the only ones that still read step j's values, had read them before.
+// these, the only ones that still read step j's values, had read them before.  A diagonal goes
+// to the CTAs that hold a remaining row, an entry l_a to those that hold one besides the
+// pivot row: there, each remaining row waits for all values of the step.
 // k = 128: 240 us; with the pivot row fetched from its owner between CTA and cluster barriers
 // 300 us, as a one-CTA factorisation 399 us.
 constexpr int kXC = 8;
@@ -505,6 +510,7 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
   // them then remains, whose next values wait for the extra warp's, so that no buffer is
   // written again before the extra warp has read it.  The last row does its work itself.
   int mine = c < kx ? (kx - c + kXC - 1) / kXC : 0;
+  int left = lane < kXC && lane < kx ? (kx - lane + kXC - 1) / kXC : 0;   // the same of CTA `lane`
   bool expired = false;
   for (int j = 0; j < kx && (has || (scalar && mine > 1)); ++j) {
     const bool solo = mine == 1;
@@ -521,7 +527,7 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
       for (int i = 0; i < NS; ++i)
         if (i == (a >> 5)) ds = S[i];
       ds = __shfl_sync(0xffffffffu, ds, a & 31);
-      if (lane < kXC)
+      if (left > 0)
         push_pair(&kbuf[par][a], &kbar[par], lane, (unsigned)__double2loint(ds), (unsigned)__double2hiint(ds));
     }
     expired = !bar_wait(&kbar[par], ph);
@@ -554,6 +560,7 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
       break;
     }
     const int p = (int)(pi & 0xffffu);
+    if (p % kXC == lane) --left;
     if (nq == 0) {                                    // the column in place j moves to the pivot's
 #pragma unroll
       for (int i = 0; i < NS; ++i)
@@ -578,7 +585,7 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
         rl = sbuf[par];
       }
       const double l = (a == p ? piv : rs) * rl;
-      if (lane < kXC)
+      if (left > 0)
         push_pair(&rbuf[par][a], &rbar[par], lane, (unsigned)__double2loint(l), (unsigned)__double2hiint(l));
       if (lane == 0) Lmine[wid * kx + j] = l;
       if (a == p) {                                   // this row is the pivot row
@@ -762,6 +769,7 @@ constexpr int kInvIters = 3;
 //   row j + 1 to all CTAs.  With p and row j + 1 of all rows: K = t/2 p.v, w = p - K v; it
 //   updates its row and the copy of row j + 1, which is the next x.  The warp of row j
 //   records the step (reflector, d_j, e_j) and is done.
+//   Only CTAs with a row g > j get the values of step j: the warps of those rows wait for all.
 //   The slots are double-buffered by the parity of the step: a warp sends in step j + 2 only
 //   after the values of step j + 1 of every row >= j + 1 have arrived, and the warps of
 //   those rows, the only ones that still read, sent them after they had read step j's.
@@ -814,6 +822,7 @@ eig32_cl_kernel(int n, DW w) {
   float* V = w.A32;                                   // reflector rows for backtr_kernel
   float *gd = w.T3, *ge = w.T3 + n;                   // d and e, by the warps of their rows
   const bool arms = g < r && g + kEC >= r;            // the CTA's last row: its warp leaves last
+  const int last = lane < kEC && lane < r ? lane + (r - 1 - lane) / kEC * kEC : -1;   // that row of CTA `lane`
   bool ok = true;
   for (int j = 0; j + 2 < r && j <= g && g < r; ++j) {
     const int j1 = j + 1, par = j & 1;
@@ -855,7 +864,7 @@ eig32_cl_kernel(int n, DW w) {
       s = fmaf(A[i], v[i], s);
     }
     s = warp_sumf(s);
-    if (lane < kEC) push_pair(&buf[par][g], &bars[par], lane, __float_as_uint(t * s), __float_as_uint(a1));
+    if (last > j) push_pair(&buf[par][g], &bars[par], lane, __float_as_uint(t * s), __float_as_uint(a1));
     if (g == j) {
       // this row's step: the reflector and the tridiagonal entries; no one reads this row again
 #pragma unroll
