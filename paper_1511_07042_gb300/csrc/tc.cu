@@ -784,6 +784,7 @@ gram_tc_kernel(const TI* __restrict__ X, const TI* __restrict__ Y, int n, int k,
   workers_scan_sync(&sh.abort_flag);
   if (tid < kNB) sh.run[0][tid] = sh.exB[0][tid];
   int g = 0, w = 0;
+  bool left = false;        // the same in every worker: the flag itself may rise at any time
   for (int w0 = r0; w0 < r1; w0 += kWindow, ++w) {
     const int w1 = min(r1, w0 + kWindow);
     const int nsub = (w1 - w0 + kKsub - 1) / kKsub;
@@ -817,9 +818,10 @@ gram_tc_kernel(const TI* __restrict__ X, const TI* __restrict__ Y, int n, int k,
       }
       hand_over(sh, b);
     }
-    if (workers_scan_sync(&sh.abort_flag)) break;    // the exponents of the next window are complete
+    left = workers_scan_sync(&sh.abort_flag);        // the exponents of the next window are complete
+    if (left) break;
   }
-  if (w > 0 && !sh.abort_flag) {
+  if (w > 0 && !left) {
     wait_sub(sh, g - 1);
     __syncwarp();
     fence_after();
@@ -1090,6 +1092,7 @@ expand_tc_kernel(const TI* __restrict__ Z, const TI* __restrict__ X, const unsig
     fence_before();
   };
   int g = 0, t = 0, ptile = -1, pjb = 0;     // the block whose sums are still in tensor memory
+  bool left = false;                         // the same in every worker, as in the Gram kernel
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++t) {
     const int row = tile * 128 + rl;
     const int E = sh.exA[t & 3][rl];
@@ -1130,9 +1133,10 @@ expand_tc_kernel(const TI* __restrict__ Z, const TI* __restrict__ X, const unsig
       ptile = tile;
       pjb = jbi;
     }
-    if (workers_scan_sync(&sh.abort_flag)) break;    // the exponents of the next tile are complete
+    left = workers_scan_sync(&sh.abort_flag);        // the exponents of the next tile are complete
+    if (left) break;
   }
-  if (ptile >= 0 && !sh.abort_flag) {
+  if (ptile >= 0 && !left) {
     wait_sub(sh, g - 1);
     __syncwarp();
     fence_after();
