@@ -340,10 +340,10 @@ bmg_status bmg_gram_tc_f32(const float* X, const float* Y, int n, int k, int ld,
 
 /* Test of the bounded waits inside the tensor-core kernels (every wait on an
  * mbarrier gives up after a clock limit, frees the kernel's tensor memory and raises
- * an error flag).  Runs a float64 Gram of a zero 4096 x 64 block whose MMA-issuing warp
- * issues nothing, with a wait limit of about 1 ms, so that the waits for the MMA
- * commits expire.  Returns BMG_ERR_TIMEOUT, as a product call after such an expiry
- * does; BMG_ERR_CUDA if the waits did not expire.  The CUDA context stays usable
+ * an error flag).  Runs a float64 Gram and an expansion of zero 4096 x 64 blocks whose
+ * MMA-issuing warp issues nothing, with a wait limit of about 1 ms, so that the waits for
+ * the MMA commits expire inside the kernels' loops.  Returns BMG_ERR_TIMEOUT, as a product
+ * call after such an expiry does; BMG_ERR_CUDA if the waits did not expire there.  The CUDA context stays usable
  * (the tests run a normal Gram after it).  Allocates and frees its own buffers.
  * Synchronous.                                                                      */
 bmg_status bmg_tc_timeout_selftest(void* stream);

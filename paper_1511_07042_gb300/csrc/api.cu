@@ -547,18 +547,30 @@ extern "C" bmg_status bmg_gram_tc_f32(const float* X, const float* Y, int n, int
   });
 }
 
-// Test of the tensor-core kernels' bounded waits: a Gram whose waits are made to
-// expire (gram_tc_timeout_selftest).  Returns what a product call returns after such
-// an expiry, BMG_ERR_TIMEOUT, once the kernel has returned; the context stays usable.
+// Test of the tensor-core kernels' bounded waits: a Gram and an expansion whose waits are
+// made to expire inside their loops.  Returns what a product call returns after such an
+// expiry, BMG_ERR_TIMEOUT, once the kernels have returned; the context stays usable.
 extern "C" bmg_status bmg_tc_timeout_selftest(void* stream) {
   return guarded([&] {
     cudaStream_t s = (cudaStream_t)stream;
-    DBuf<double> X((size_t)4096 * 64), G((size_t)64 * 64);
-    Workspace ws(sizeof(double) * (size_t)gram_tc_parts(4096, 64) * 64 * 64, s);
-    BMG_CUDA(cudaMemsetAsync(X.get(), 0, sizeof(double) * 4096 * 64, s));
+    const size_t nk = (size_t)4096 * 64, kk = 64 * 64;
+    DBuf<double> X(nk), U(nk), G(kk), C(kk);
+    Workspace ws(std::max(sizeof(double) * kTcSelftestParts * kk, expand_tc_scratch_bytes(64)), s);
+    BMG_CUDA(cudaMemsetAsync(X.get(), 0, sizeof(double) * nk, s));
+    BMG_CUDA(cudaMemsetAsync(C.get(), 0, sizeof(double) * kk, s));
+    volatile int* flag = ws.flag();
     gram_tc_timeout_selftest(X.get(), G.get(), ws.get<double>(), ws.flag(), s);
-    finish_tc(ws, s);
-    fail(BMG_ERR_CUDA, "tc timeout self-test: the bounded waits did not expire");
+    BMG_CUDA(cudaStreamSynchronize(s));
+    const int gram_left = *flag;
+    *flag = 0;
+    expand_tc_timeout_selftest(X.get(), C.get(), U.get(), ws.get<unsigned char>(), ws.flag(), s);
+    BMG_CUDA(cudaStreamSynchronize(s));
+    const int expand_left = *flag;
+    ws.idle();
+    if (gram_left != 3 || expand_left != 3)
+      fail(BMG_ERR_CUDA, "tc timeout self-test: the bounded waits did not expire in the loops (Gram " +
+                             std::to_string(gram_left) + ", expansion " + std::to_string(expand_left) + ")");
+    fail(BMG_ERR_TIMEOUT, "a bounded wait in a tensor-core kernel expired");
   });
 }
 

@@ -341,9 +341,12 @@ void gram_tc(const TI* X, const TI* Y, int n, int k, int ld, double* G, double* 
 template <typename TI>
 void expand_tc(const TI* Zf, const TI* X, const double* Yx, int n, int k, int ld, int ldy, TI* U,
                unsigned char* scratch, int* err, cudaStream_t s);
-// A float64 Gram of the zero 4096 x 64 block X whose bounded waits are made to expire
-// (see tc.cu); raises *err.
+// A float64 Gram and an expansion (X, U: 4096 x 64, Yx: 64 x 64, zeros) whose bounded waits are
+// made to expire inside their loops (see tc.cu); raise bits 0 and 1 of *err.
+constexpr int kTcSelftestParts = 4;
 void gram_tc_timeout_selftest(const double* X, double* G, double* partial, int* err, cudaStream_t s);
+void expand_tc_timeout_selftest(const double* X, const double* Yx, double* U, unsigned char* scratch, int* err,
+                                cudaStream_t s);
 template <typename T>
 void eig_residuals(const T* AU, const T* MU, const T* U, const double* lam, int n, int k, int ld,
                    double* partial, int nparts, double* out, cudaStream_t s);

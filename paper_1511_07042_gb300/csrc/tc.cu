@@ -124,7 +124,7 @@ __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::aft
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // Waits for the completion of the phase with the given parity; false after `limit`
-// clocks without it (kWaitCycles, about 2 s, except in the timeout self-test).
+// clocks without it (kWaitCycles, about 2 s, except in the timeout self-tests).
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long limit) {
   const long long t0 = clock64();
   while (true) {
@@ -456,7 +456,7 @@ template <> struct Epi<float> {
   }
 };
 
-// Launch controls: the limit of every bounded wait, and (timeout self-test only) an
+// Launch controls: the limit of every bounded wait, and (timeout self-tests only) an
 // MMA warp that issues nothing, so that the workers' waits for commits expire.
 struct TcCtl {
   long long wait_cycles;
@@ -534,9 +534,10 @@ __device__ __forceinline__ void tc_setup(TcShared& sh, unsigned char* smem, int 
 
 // End of a tensor-core kernel, reached by every thread.  The issuing thread first
 // waits (bounded) for the last commit of each stage, so that no MMA is in flight when
-// the tensor memory is freed (after a timed-out wait the MMAs may still run).
+// the tensor memory is freed (after a timed-out wait the MMAs may still run).  *err: bit 0 a
+// wait expired, bit 1 the workers and scan warps left their loops for it (left).
 template <int T>
-__device__ __forceinline__ void tc_teardown(TcShared& sh, int issued, int* err) {
+__device__ __forceinline__ void tc_teardown(TcShared& sh, int issued, int* err, bool left = false) {
   if (threadIdx.x == kWorkers) {
     for (int b = 0; b < 2; ++b) {
       const int uses = (issued - b + 1) / 2;   // commits made on stage b
@@ -549,7 +550,7 @@ __device__ __forceinline__ void tc_teardown(TcShared& sh, int issued, int* err) 
     fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sh.tmem_slot), "r"(tmem_cols<T>()));
   }
-  if (sh.abort_flag && threadIdx.x == 0) atomicExch(err, 1);
+  if (sh.abort_flag && threadIdx.x == 0) atomicOr(err, left ? 3 : 1);
 }
 
 // Waits (every worker) for the commit of sub-chunk gi; raises the shared abort flag
@@ -841,7 +842,7 @@ gram_tc_kernel(const TI* __restrict__ X, const TI* __restrict__ Y, int n, int k,
                      : wide_value(R[q], e_run + run[c_base + q] + off);
     }
   }
-  tc_teardown<T>(sh, 0, err);
+  tc_teardown<T>(sh, 0, err, left);
 }
 
 // ------------------------------------------------------------ expand ----------
@@ -1143,7 +1144,7 @@ expand_tc_kernel(const TI* __restrict__ Z, const TI* __restrict__ X, const unsig
     readback(t - 1, ptile, pjb);
   }
   workers_sync();
-  tc_teardown<T>(sh, 0, err);
+  tc_teardown<T>(sh, 0, err, left);
 }
 
 int num_sms() {
@@ -1208,19 +1209,10 @@ void gram_tc(const TI* X, const TI* Y, int n, int k, int ld, double* G, double* 
   gram_tc_launch<TI>(X, Y, n, k, ld, G, partial, nparts, err, s, sym, TcCtl{kWaitCycles, 0});
 }
 
-// The bounded waits of the tensor-core kernels, made to run out: a float64 Gram of a
-// zero 4096 x 64 block whose MMA warp issues nothing, with waits of about 1 ms.  The
-// workers' waits for the commits expire; the kernel must raise *err, free its tensor
-// memory and return.  Buffers are the caller's (partial: gram_tc_parts(4096, 64) * 64^2
-// doubles).
-void gram_tc_timeout_selftest(const double* X, double* G, double* partial, int* err, cudaStream_t s) {
-  gram_tc_launch<double>(X, X, 4096, 64, 64, G, partial, gram_tc_parts(4096, 64), err, s, true,
-                         TcCtl{2000000LL, 1});
-}
-
+namespace {
 template <typename TI>
-void expand_tc(const TI* Zf, const TI* X, const double* Yx, int n, int k, int ld, int ldy, TI* U,
-               unsigned char* scratch, int* err, cudaStream_t s) {
+void expand_tc_launch(const TI* Zf, const TI* X, const double* Yx, int n, int k, int ld, int ldy, TI* U,
+                      unsigned char* scratch, int* err, cudaStream_t s, int ctas, TcCtl ctl) {
   if (k > kTcMaxK) fail(BMG_ERR_INVALID_ARG, "expand_tc: k > 128");
   constexpr int S = Digits<TI>::S;
   const int njb = (k + kNB - 1) / kNB, nsub = (k + kKsub - 1) / kKsub;
@@ -1231,15 +1223,35 @@ void expand_tc(const TI* Zf, const TI* X, const double* Yx, int n, int k, int ld
   // few tiles: a CTA per tile and column block (twice the SMs at work); many: the blocks of
   // a tile in one CTA, which then reads the X tile from DRAM and forms its exponents once
   const int ntiles = (n + 127) / 128;
-  const dim3 grid(std::min(ntiles, num_sms()), ntiles * njb <= num_sms() ? njb : 1);
+  const dim3 grid(std::min(ntiles, ctas), ntiles * njb <= ctas ? njb : 1);
   const int vec = aligned16(X) && aligned16(U) && aligned16(Zf) && (size_t)ld * sizeof(TI) % 16 == 0;
   prof_begin(KC_EXPAND, s);
   expand_prep_kernel<TI><<<dim3(njb, nsub), kPrepThreads, 0, s>>>(Yx, k, ldy, scratch, gexp);
   check_launch("expand_prep_kernel");
-  expand_tc_kernel<TI><<<grid, kTcThreads, smem, s>>>(Zf, X, scratch, gexp, n, k, ld, nsub, njb, U, vec, err,
-                                                       TcCtl{kWaitCycles, 0});
+  expand_tc_kernel<TI><<<grid, kTcThreads, smem, s>>>(Zf, X, scratch, gexp, n, k, ld, nsub, njb, U, vec, err, ctl);
   check_launch("expand_tc_kernel");
   prof_end(KC_EXPAND, s, 3.0 * sizeof(TI) * n * ld + 8.0 * k * k, 2.0 * n * k * k);
+}
+}  // namespace
+
+template <typename TI>
+void expand_tc(const TI* Zf, const TI* X, const double* Yx, int n, int k, int ld, int ldy, TI* U,
+               unsigned char* scratch, int* err, cudaStream_t s) {
+  expand_tc_launch<TI>(Zf, X, Yx, n, k, ld, ldy, U, scratch, err, s, num_sms(), TcCtl{kWaitCycles, 0});
+}
+
+// The bounded waits of the tensor-core kernels, made to run out: float64 products of zero
+// 4096 x 64 blocks whose MMA warp issues nothing, with waits of about 1 ms.  A part of the Gram
+// has four windows of eight sub-chunks and a CTA of the expansion eight tiles of two, so that
+// the waits for a stage in use expire inside the loops and the warps leave these together; the
+// kernels must raise both bits of *err, free their tensor memory and return.
+// partial: kTcSelftestParts * 64^2 doubles.
+void gram_tc_timeout_selftest(const double* X, double* G, double* partial, int* err, cudaStream_t s) {
+  gram_tc_launch<double>(X, X, 4096, 64, 64, G, partial, kTcSelftestParts, err, s, true, TcCtl{2000000LL, 1});
+}
+void expand_tc_timeout_selftest(const double* X, const double* Yx, double* U, unsigned char* scratch, int* err,
+                                cudaStream_t s) {
+  expand_tc_launch<double>(nullptr, X, Yx, 4096, 64, 64, 64, U, scratch, err, s, 4, TcCtl{2000000LL, 1});
 }
 
 template void gram_tc<double>(const double*, const double*, int, int, int, double*, double*, int, int*, cudaStream_t,
