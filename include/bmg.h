@@ -368,10 +368,23 @@ bmg_status bmg_expand_f32(const float* Z, const float* X, const double* Yx, int 
  * tridiagonal start refined to FP64 accuracy.  (bmg_solve factors the enriched
  * Mhat in block form, reusing the factor of its coarse-space block.)
  * theta [k], Y [n][k] device; Y^T Mhat Y = I.  rank_out (device int or NULL)
- * receives the kept rank.  Errors: BMG_ERR_INVALID_ARG; a rank below k is
- * reported through bmg_solve as BMG_ERR_SINGULAR.                               */
+ * receives the kept rank; with a rank below k the outputs past it are not set
+ * (bmg_solve reports it as BMG_ERR_SINGULAR).  Where the refinement does not
+ * converge (error estimate above 1e-6), the solve is repeated, twice from other
+ * start vectors and once from an FP64 Jacobi start (some 10 ms).  Errors:
+ * BMG_ERR_INVALID_ARG; BMG_ERR_NONFINITE when no attempt converged (matrices with
+ * Inf or NaN); BMG_ERR_TIMEOUT when a bounded wait inside the kernels expired.
+ * Synchronous.                                                                  */
 bmg_status bmg_dense_eig(const double* Ahat, const double* Mhat, int n, double sigma,
                          int k, double* theta, double* Y, int* rank_out, void* stream);
+/* For tests: attempt number `start` of bmg_dense_eig alone (which takes 0, 1, 2, 3
+ * in turn); err (host) receives the error estimate, however large.             */
+bmg_status bmg_dense_eig_attempt(const double* Ahat, const double* Mhat, int n, double sigma,
+                                 int k, double* theta, double* Y, int start, double* err,
+                                 void* stream);
+/* Test of the bounded waits of the eigensolve's kernels, as bmg_tc_timeout_selftest:
+ * BMG_ERR_TIMEOUT when they expired, BMG_ERR_CUDA otherwise.  Synchronous.       */
+bmg_status bmg_dense_timeout_selftest(void* stream);
 
 /* The same product as bmg_gram for callers that must not allocate device memory:
  * a framework that has already reserved all device memory for its own pool, a

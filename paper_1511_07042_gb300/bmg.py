@@ -91,6 +91,8 @@ def _load():
         "bmg_expand": (i, [vp, vp, vp, i, i, i, i, vp, i, vp]),
         "bmg_expand_f32": (i, [vp, vp, vp, i, i, i, i, vp, i, vp]),
         "bmg_dense_eig": (i, [vp, vp, i, d, i, vp, vp, vp, vp]),
+        "bmg_dense_eig_attempt": (i, [vp, vp, i, d, i, vp, vp, i, C.POINTER(d), vp]),
+        "bmg_dense_timeout_selftest": (i, [vp]),
         "bmg_profile_enable": (i, [i]),
         "bmg_profile_reset": (i, []),
         "bmg_profile_read": (i, [i, P(C.c_double), P(C.c_longlong), P(C.c_double), P(C.c_double)]),
@@ -420,3 +422,16 @@ def gram_noalloc(X, Y, k, G):
 def dense_eig(Ahat, Mhat, sigma, k, theta, Y, rank=None):
     _check(LIB.bmg_dense_eig(_ptr(Ahat), _ptr(Mhat), Ahat.shape[0], float(sigma), k, _ptr(theta),
                              _ptr(Y), _ptr(rank), _stream()))
+
+
+def dense_eig_attempt(Ahat, Mhat, sigma, k, theta, Y, start):
+    """Error estimate of one attempt of dense_eig from start vectors `start`."""
+    err = C.c_double()
+    _check(LIB.bmg_dense_eig_attempt(_ptr(Ahat), _ptr(Mhat), Ahat.shape[0], float(sigma), k, _ptr(theta),
+                                     _ptr(Y), int(start), C.byref(err), _stream()))
+    return err.value
+
+
+def dense_timeout_selftest():
+    """Status code of bmg_dense_timeout_selftest (BMG_ERR_TIMEOUT when the waits expired)."""
+    return int(LIB.bmg_dense_timeout_selftest(_stream()))

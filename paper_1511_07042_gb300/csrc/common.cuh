@@ -90,7 +90,8 @@ void DBuf<T>::alloc(size_t count) {
 // for the stream unless idle() was called after a synchronisation.  The pool keeps at most
 // kPoolBytes per device, is emptied by every bmg_destroy and when a device allocation
 // fails, and takes calls from several threads.  flag() is a pinned host word that the
-// call's kernels may raise; it is zero on construction.
+// call's kernels may raise; it is zero on construction.  value() is a pinned host double that
+// they may write.
 class Workspace {
  public:
   Workspace(size_t bytes, cudaStream_t s);
@@ -99,6 +100,7 @@ class Workspace {
   Workspace& operator=(const Workspace&) = delete;
   template <typename T> T* get() const { return static_cast<T*>(ptr_); }
   int* flag() const { return flag_; }
+  double* value() const { return reinterpret_cast<double*>(flag_ + 2); }
   void idle() { idle_ = true; }
 
  private:
@@ -368,9 +370,26 @@ constexpr double kDropFP32 = 1e-5;
 // sel_first < 0: the k pairs of smallest |theta| (index-updating); >= 0: positions
 // sel_first .. sel_first + k - 1 of the ascending values (index-fixed; moved down when
 // past the top), ordered by (|theta|, theta, index) like the former.
-// salt: set of start vectors of the inverse iteration (another one for a second attempt).
+// salt: the attempt, 0 for the first.
+// quality: the error estimate of the refinement, or kEigExpired when a bounded wait of the
+// cluster exchanges expired.  The refinement diverges when two start vectors of a tight cluster
+// come out of the float32 inverse iteration nearly parallel (about one solve in 300 from random
+// blocks, at any rounding of the products), and it does not converge for groups of more than 40
+// pairs closer than 1e-3 of the largest.  Callers take an estimate up to kEigMaxError and repeat
+// the solve, kEigAttempts in all: with salts 1 and 2 from other start vectors, with the last one
+// from an FP64 start.
+// host_rank: mapped host word that receives the rank too.
+constexpr double kEigMaxError = 1e-6, kEigExpired = -1.0;
+constexpr int kEigAttempts = 4;
+// Limit of the bounded waits (about a second), and (self-test only) a row of the factorisation
+// and of the tridiagonalisation that sends nothing, so that the others' waits expire.
+struct ExchangeCtl {
+  long long wait_cycles = 2000000000LL;
+  int mute_factor = -1, mute_tridiag = -1;
+};
 void dense_eig(const double* Ahat, const double* Mhat, int n, double sigma, int k,
                double* theta, double* Y, int* rank, double* work, double* quality, double drop_tol,
-               int nq, cudaStream_t s, int sel_first = -1, int salt = 0);
+               int nq, cudaStream_t s, int sel_first = -1, int salt = 0, int* host_rank = nullptr,
+               ExchangeCtl ctl = {});
 size_t dense_work_doubles(int n);
 }  // namespace bmg

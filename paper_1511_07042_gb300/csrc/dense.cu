@@ -423,9 +423,9 @@ __device__ __forceinline__ void bar_expect(unsigned long long* bar, unsigned byt
                "r"(bytes)
                : "memory");
 }
-// Waits for the phase of the given parity; false after about a second (the callers then
-// leave their loops, and the solve reports the result as not finite).
-__device__ __forceinline__ bool bar_wait(unsigned long long* bar, unsigned parity) {
+// Waits for the phase of the given parity; false after `limit` clocks (the callers then leave
+// their loops and raise w.misc[2], and the call reports the expired wait).
+__device__ __forceinline__ bool bar_wait(unsigned long long* bar, unsigned parity, long long limit) {
   const long long t0 = clock64();
   while (true) {
     unsigned done;
@@ -436,7 +436,7 @@ __device__ __forceinline__ bool bar_wait(unsigned long long* bar, unsigned parit
         : "r"(smem_u32(bar)), "r"(parity)
         : "memory");
     if (done) return true;
-    if (clock64() - t0 > 2000000000LL) return false;
+    if (clock64() - t0 > limit) return false;
   }
 }
 
@@ -464,7 +464,7 @@ __device__ __forceinline__ bool bar_wait(unsigned long long* bar, unsigned parit
 constexpr int kXC = 8;
 template <int NS>
 __global__ void __cluster_dims__(kXC, 1, 1) __launch_bounds__(32 * (32 * NS / kXC + 1))
-xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
+xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol, ExchangeCtl ctl) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   constexpr int nrow = 32 * NS / kXC;                 // rows of a CTA, one warp each
@@ -479,7 +479,10 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
   const int c = (int)cl.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   if (nq > 0 && w.qflag[0] != 1) {                    // the same decision in every CTA
-    if (c == 0 && tid == 0) *w.rank = 0;
+    if (c == 0 && tid == 0) {
+      *w.rank = 0;
+      w.misc[2] = 0.0;
+    }
     return;
   }
   // pivot order and reciprocal roots through global memory, then the rank
@@ -499,7 +502,7 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
   if (tid == 0) {
     for (int q = 0; q < 2; ++q) { bar_init(&kbar[q]); bar_init(&rbar[q]); bar_init(&sbar[q]); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    if (c == 0) { grank[0] = kx; grank[1] = 0; }
+    if (c == 0) { grank[0] = kx; grank[1] = 0; w.misc[2] = 0.0; }
   }
   cl.sync();
   unsigned gone = 0u;                                 // eliminated columns of this lane, a bit per slot
@@ -527,10 +530,10 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
       for (int i = 0; i < NS; ++i)
         if (i == (a >> 5)) ds = S[i];
       ds = __shfl_sync(0xffffffffu, ds, a & 31);
-      if (left > 0)
+      if (left > 0 && a != ctl.mute_factor)
         push_pair(&kbuf[par][a], &kbar[par], lane, (unsigned)__double2loint(ds), (unsigned)__double2hiint(ds));
     }
-    expired = !bar_wait(&kbar[par], ph);
+    expired = !bar_wait(&kbar[par], ph, ctl.wait_cycles);
     if (__any_sync(0xffffffffu, expired)) { expired = true; break; }
     // the pivot: largest key, then smallest index
     unsigned khi[NS], klo[NS], m1 = 0u;
@@ -580,7 +583,7 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
       if (solo) {
         rl = rsqrt_nr(piv);
       } else {
-        expired = !bar_wait(&sbar[par], ph);
+        expired = !bar_wait(&sbar[par], ph, ctl.wait_cycles);
         if (__any_sync(0xffffffffu, expired)) { expired = true; break; }
         rl = sbuf[par];
       }
@@ -592,7 +595,7 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
         if (lane == 0) { gperm[j] = p; grl[j] = rl; }
         break;
       }
-      expired = !bar_wait(&rbar[par], ph);
+      expired = !bar_wait(&rbar[par], ph, ctl.wait_cycles);
       if (__any_sync(0xffffffffu, expired)) { expired = true; break; }
       if ((p & 31) == lane) gone |= 1u << (p >> 5);
 #pragma unroll
@@ -605,7 +608,10 @@ xfactor_cl_kernel(int n, int nq, int kx, DW w, double drop_tol) {
     if (scalar && (p & 31) == lane) gone |= 1u << (p >> 5);
     if (p % kXC == c) --mine;
   }
-  if (expired && lane == 0) grank[1] = 1;
+  if (expired && lane == 0) {
+    grank[1] = 1;
+    w.misc[2] = 1.0;
+  }
   cl.sync();                                          // pivots and rank complete; no more sends
   const int rx = __ldcg(grank + 1) ? 0 : __ldcg(grank);
   for (int i = tid; i < kx; i += kXThreads) done[i] = 0;
@@ -782,7 +788,7 @@ constexpr int kInvIters = 3;
 constexpr int kEC = 8;
 template <int NS>
 __global__ void __cluster_dims__(kEC, 1, 1) __launch_bounds__(32 * 32 * NS / kEC)
-eig32_cl_kernel(int n, DW w) {
+eig32_cl_kernel(int n, DW w, ExchangeCtl ctl) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   constexpr int nwarps = 32 * NS / kEC;               // rows of a CTA, one warp each
@@ -864,7 +870,7 @@ eig32_cl_kernel(int n, DW w) {
       s = fmaf(A[i], v[i], s);
     }
     s = warp_sumf(s);
-    if (last > j) push_pair(&buf[par][g], &bars[par], lane, __float_as_uint(t * s), __float_as_uint(a1));
+    if (last > j && g != ctl.mute_tridiag) push_pair(&buf[par][g], &bars[par], lane, __float_as_uint(t * s), __float_as_uint(a1));
     if (g == j) {
       // this row's step: the reflector and the tridiagonal entries; no one reads this row again
 #pragma unroll
@@ -884,7 +890,7 @@ eig32_cl_kernel(int n, DW w) {
     for (int i = 0; i < NS; ++i)
       if (i == (g >> 5)) vgs = v[i];
     const float vg = __shfl_sync(0xffffffffu, vgs, g & 31);
-    ok = bar_wait(&bars[par], (unsigned)(j >> 1) & 1u);
+    ok = bar_wait(&bars[par], (unsigned)(j >> 1) & 1u, ctl.wait_cycles);
     if (!__all_sync(0xffffffffu, ok)) {
       ok = false;
       break;
@@ -918,6 +924,7 @@ eig32_cl_kernel(int n, DW w) {
       if (t != 0.f) A[i] = A[i] - __fadd_rn(__fmul_rn(vg, wi), __fmul_rn(wg, v[i]));
     }
   }
+  if (!ok && lane == 0) w.misc[2] = 1.0;
   // the last entries: rows r - 2 and r - 1 hold them
   if (g < r && g + 2 >= r) {
 #pragma unroll
@@ -1571,22 +1578,22 @@ constexpr int kClThreads = 256;
 constexpr size_t kClSmem = sizeof(double) * 5 * kMaxCluster * kMaxCluster + sizeof(float) * 2 * kMaxCluster * kMaxCluster;
 // Cyclic Jacobi sweeps (round-robin pairing, mm/2 rotations per round) on the mm x mm
 // matrix A, accumulating the rotations into V, until off(A) <= tol fro(A) or `sweeps`
-// sweeps; T is the arithmetic (float or double).
-template <typename T>
+// sweeps; T is the arithmetic (float or double), NT the threads of the CTA.
+template <typename T, int NT>
 __device__ void jacobi_sweeps(T* A, T* V, int mm, int sweeps, T tol, T* ccs_c, T* ccs_s, int* cpr_p,
                               int* cpr_q, int* cpr_r, T* red) {
   const int tid = threadIdx.x;
   const int m2 = (mm % 2 == 0) ? mm : mm + 1;
   for (int sweep = 0; sweep < sweeps; ++sweep) {
     T off = 0, fro = 0;
-    for (int q = tid; q < mm * mm; q += kClThreads) {
+    for (int q = tid; q < mm * mm; q += NT) {
       const T v = A[q];
       fro += v * v;
       if (q / mm != q % mm) off += v * v;
     }
     off = block_sum<T>(off, red);
     fro = block_sum<T>(fro, red);
-    if (off <= tol * fro || fro == T(0)) break;
+    if (!(off > tol * fro)) break;        // converged, or not finite
     for (int step = 0; step < m2 - 1; ++step) {
       if (tid < m2 / 2) {
         const int i = tid;
@@ -1630,7 +1637,7 @@ __device__ void jacobi_sweeps(T* A, T* V, int mm, int sweeps, T tol, T* ccs_c, T
       // partner (q = mm) has no rotation.  The fused forms are written out: a product rounded
       // the other way would turn the vectors of equal eigenvalues
       const int half = m2 / 2, blocks = half * half;
-      for (int it = tid; it < blocks + half * mm; it += kClThreads) {
+      for (int it = tid; it < blocks + half * mm; it += NT) {
         if (it < blocks) {
           const int i = it / half, j = it - i * half;
           const bool ri = cpr_r[i], rj = cpr_r[j];
@@ -1741,7 +1748,7 @@ cluster_kernel(int n, DW w) {
     fV[q] = (a == e) ? 1.f : 0.f;
   }
   __syncthreads();
-  jacobi_sweeps<float>(fA, fV, mm, 12, 1e-13f, fcs_c, fcs_s, cpr_p, cpr_q, cpr_r, redf);
+  jacobi_sweeps<float, kClThreads>(fA, fV, mm, 12, 1e-13f, fcs_c, fcs_s, cpr_p, cpr_q, cpr_r, redf);
   // V1 = V0 (3 I - V0^T V0) / 2
   for (int q = tid; q < mm * mm; q += kClThreads) {
     const int a = q / mm, e = q % mm;
@@ -1762,13 +1769,33 @@ cluster_kernel(int n, DW w) {
     }
   }
   __syncthreads();
-  jacobi_sweeps<double>(cA, cV, mm, 10, 1e-32, ccs_c, ccs_s, cpr_p, cpr_q, cpr_r, red);
+  jacobi_sweeps<double, kClThreads>(cA, cV, mm, 10, 1e-32, ccs_c, ccs_s, cpr_p, cpr_q, cpr_r, red);
   for (int q = tid; q < mm * mm; q += kClThreads) {
     const int a = q / mm, e = q % mm;
     double sacc = 0.0;
     for (int u = 0; u < mm; ++u) sacc += cK[a * mm + u] * cV[u * mm + e];
     w.E[idx[a] * n + idx[e]] = sacc - (a == e ? 1.0 : 0.0);
   }
+}
+
+// Start of the last attempt: W = eigenvectors of sym(T) by cyclic Jacobi in FP64, the matrix
+// and the rotations in w.P and w.Z, one CTA.  Slow (n = 170: 86 ms), but it depends on no
+// start vectors, and the refinement needs nothing from it for groups of more than kMaxCluster
+// pairs, which the cluster step does not diagonalise.
+__global__ void __launch_bounds__(kBig) jacobi_start_kernel(int n, DW w) {
+  __shared__ double cs[kMaxDense / 2], sn[kMaxDense / 2], red[32];
+  __shared__ int rp[kMaxDense / 2], rq[kMaxDense / 2], rr[kMaxDense / 2];
+  const int r = *w.rank;
+  for (int t = threadIdx.x; t < r * r; t += kBig) {
+    const int i = t / r, j = t - i * r;
+    w.P[t] = 0.5 * (w.T[i * n + j] + w.T[j * n + i]);
+    w.Z[t] = i == j ? 1.0 : 0.0;
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < r * r; t += kBig) w.T[(t / r) * n + t % r] = w.P[t];
+  __syncthreads();
+  jacobi_sweeps<double, kBig>(w.P, w.Z, r, 40, 1e-28, cs, sn, rp, rq, rr, red);
+  for (int t = threadIdx.x; t < r * r; t += kBig) w.W[(t / r) * n + t % r] = w.Z[t];
 }
 
 // ------------------------------------------- 5. selection and back-transform --
@@ -1783,7 +1810,7 @@ __global__ void select_kernel(int k, int n, const double* acc, DW w, double* __r
   const double2 nrm = part_sums(w.part, n, red);
   if (threadIdx.x == 0) {
     const double amax = acc_max(acc);
-    w.misc[1] = (amax > 0.0) ? sqrt(nrm.x) / amax + sqrt(nrm.y) : sqrt(nrm.y);
+    w.misc[1] = sqrt(nrm.x) / (amax > 0.0 ? amax : 1.0) + sqrt(nrm.y);   // (NaN values leave amax 0)
   }
   __syncthreads();
   // order by (|lam|, lam, index) through integer keys: the magnitude's bits, then a
@@ -1882,9 +1909,11 @@ backsub_kernel(int n, int k, DW w, double* __restrict__ Y) {
   }
 }
 
-__global__ void copy_out_kernel(DW w, int* rank_out, double* quality) {
+// (rank also to host_rank, a mapped host word, when given)
+__global__ void copy_out_kernel(DW w, int* rank_out, double* quality, int* host_rank) {
   *rank_out = *w.rank;
-  if (quality) *quality = w.misc[1];
+  if (host_rank) *host_rank = *w.rank;
+  if (quality) *quality = w.misc[2] != 0.0 ? kEigExpired : w.misc[1];
 }
 
 DW carve(double* work, int n) {
@@ -1905,7 +1934,7 @@ DW carve(double* work, int n) {
   w.d = p; p += n;
   w.rl = p; p += n;
   w.lam = p; p += n;
-  w.misc = p; p += 48;   // [0..8) scalars, [8..48) per-step norm accumulators
+  w.misc = p; p += 48;   // [1] error estimate, [2] not 0: a wait expired, [8..48) per-step norm accumulators
   w.A32 = reinterpret_cast<float*>(p); p += (nn + n) / 2 + 1;
   w.Z32 = reinterpret_cast<float*>(p); p += nn / 2 + 1;
   w.LU32 = reinterpret_cast<float*>(p); p += (5 * nn + 1) / 2 + 1;
@@ -1961,16 +1990,16 @@ void trsm(const double* Ahat, const double* Mhat, int n, double sigma, int pass,
 }
 // Pivoted Cholesky launch: a warp per row of the kx <= 32 NS new columns.
 template <int NS>
-void xfactor(int n, int nq, int kx, const DW& w, double drop_tol, cudaStream_t s) {
+void xfactor(int n, int nq, int kx, const DW& w, double drop_tol, const ExchangeCtl& ctl, cudaStream_t s) {
   const int sm = (int)((size_t)(32 * NS / kXC) * kx * sizeof(double));
   BMG_CUDA(cudaFuncSetAttribute(xfactor_cl_kernel<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
-  xfactor_cl_kernel<NS><<<kXC, 32 * (32 * NS / kXC + 1), sm, s>>>(n, nq, kx, w, drop_tol);
+  xfactor_cl_kernel<NS><<<kXC, 32 * (32 * NS / kXC + 1), sm, s>>>(n, nq, kx, w, drop_tol, ctl);
   check_launch("xfactor_cl_kernel");
 }
 // FP32 eigensolve launch: a warp per row, n <= 32 NS rows over the cluster.
 template <int NS>
-void eig32(int n, const DW& w, cudaStream_t s) {
-  eig32_cl_kernel<NS><<<kEC, 32 * 32 * NS / kEC, 0, s>>>(n, w);
+void eig32(int n, const DW& w, const ExchangeCtl& ctl, cudaStream_t s) {
+  eig32_cl_kernel<NS><<<kEC, 32 * 32 * NS / kEC, 0, s>>>(n, w, ctl);
   check_launch("eig32_cl_kernel");
 }
 void backsub(int n, int k, const DW& w, double* Y, cudaStream_t s) {
@@ -1995,7 +2024,7 @@ size_t dense_work_doubles(int n) {
 
 void dense_eig(const double* Ahat, const double* Mhat, int n, double sigma, int k, double* theta,
                double* Y, int* rank, double* work, double* quality, double drop_tol, int nq, cudaStream_t s,
-               int sel_first, int salt) {
+               int sel_first, int salt, int* host_rank, ExchangeCtl ctl) {
   if (n < 1 || n > kMaxDense || k < 1 || k > n) fail(BMG_ERR_INVALID_ARG, "dense_eig: need 1 <= k <= n <= 224");
   TraceRange trace("enriched eigensolve");
   prof_begin(KC_DENSE, s);
@@ -2022,34 +2051,40 @@ void dense_eig(const double* Ahat, const double* Mhat, int n, double sigma, int 
   schur_kernel<<<dim3(nt, nt), 64, 0, s>>>(Mhat, n, nq, kx, w);
   check_launch("schur_kernel");
   switch ((kx + 31) / 32) {
-    case 1: xfactor<1>(n, nq, kx, w, drop_tol, s); break;
-    case 2: xfactor<2>(n, nq, kx, w, drop_tol, s); break;
-    case 3: xfactor<3>(n, nq, kx, w, drop_tol, s); break;
-    case 4: xfactor<4>(n, nq, kx, w, drop_tol, s); break;
-    case 5: xfactor<5>(n, nq, kx, w, drop_tol, s); break;
-    case 6: xfactor<6>(n, nq, kx, w, drop_tol, s); break;
-    default: xfactor<7>(n, nq, kx, w, drop_tol, s); break;
+    case 1: xfactor<1>(n, nq, kx, w, drop_tol, ctl, s); break;
+    case 2: xfactor<2>(n, nq, kx, w, drop_tol, ctl, s); break;
+    case 3: xfactor<3>(n, nq, kx, w, drop_tol, ctl, s); break;
+    case 4: xfactor<4>(n, nq, kx, w, drop_tol, ctl, s); break;
+    case 5: xfactor<5>(n, nq, kx, w, drop_tol, ctl, s); break;
+    case 6: xfactor<6>(n, nq, kx, w, drop_tol, ctl, s); break;
+    default: xfactor<7>(n, nq, kx, w, drop_tol, ctl, s); break;
   }
   // 2. reduced standard matrix
   trsm(Ahat, Mhat, n, sigma, 0, w, s);
   trsm(Ahat, Mhat, n, sigma, 1, w, s);
   // 3. FP32 start: tridiagonalisation and eigenvalues (T in shared memory), inverse
   //    iteration (one CTA per cluster), back-transformation
-  switch ((n + 31) / 32) {
-    case 1: eig32<1>(n, w, s); break;
-    case 2: eig32<2>(n, w, s); break;
-    case 3: eig32<3>(n, w, s); break;
-    case 4: eig32<4>(n, w, s); break;
-    case 5: eig32<5>(n, w, s); break;
-    case 6: eig32<6>(n, w, s); break;
-    default: eig32<7>(n, w, s); break;
+  //    The last attempt takes an FP64 start instead.
+  if (salt >= kEigAttempts - 1) {
+    jacobi_start_kernel<<<1, kBig, 0, s>>>(n, w);
+    check_launch("jacobi_start_kernel");
+  } else {
+    switch ((n + 31) / 32) {
+      case 1: eig32<1>(n, w, ctl, s); break;
+      case 2: eig32<2>(n, w, ctl, s); break;
+      case 3: eig32<3>(n, w, ctl, s); break;
+      case 4: eig32<4>(n, w, ctl, s); break;
+      case 5: eig32<5>(n, w, ctl, s); break;
+      case 6: eig32<6>(n, w, ctl, s); break;
+      default: eig32<7>(n, w, ctl, s); break;
+    }
+    const size_t ism = sizeof(float) * ((size_t)n * kInvSmemMembers + kInvLuFloats);
+    BMG_CUDA(cudaFuncSetAttribute(invit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ism));
+    invit_kernel<<<n, kInvThreads, ism, s>>>(n, w, (unsigned)salt);
+    check_launch("invit_kernel");
+    backtr_kernel<<<(n + 2 * kBackWarps - 1) / (2 * kBackWarps), kBackWarps * 32, 0, s>>>(n, w);
+    check_launch("backtr_kernel");
   }
-  const size_t ism = sizeof(float) * ((size_t)n * kInvSmemMembers + kInvLuFloats);
-  BMG_CUDA(cudaFuncSetAttribute(invit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ism));
-  invit_kernel<<<n, kInvThreads, ism, s>>>(n, w, (unsigned)salt);
-  check_launch("invit_kernel");
-  backtr_kernel<<<(n + 2 * kBackWarps - 1) / (2 * kBackWarps), kBackWarps * 32, 0, s>>>(n, w);
-  check_launch("backtr_kernel");
   // 4. refinement: steps separate pairs farther apart than a floor (relative to
   //    max|lam|); the cluster step diagonalises the groups below it exactly.  Two
   //    steps from the FP32 start at its resolution (1e-3), the cluster step, and a
@@ -2089,7 +2124,7 @@ void dense_eig(const double* Ahat, const double* Mhat, int n, double sigma, int 
   select_kernel<<<1, 512, 0, s>>>(k, n, accs + 3 * nsteps, w, theta, sel_first);
   check_launch("select_kernel");
   backsub(n, k, w, Y, s);
-  copy_out_kernel<<<1, 1, 0, s>>>(w, rank, quality);
+  copy_out_kernel<<<1, 1, 0, s>>>(w, rank, quality, host_rank);
   check_launch("copy_out_kernel");
   const double nn = n;
   prof_end(KC_DENSE, s, 16.0 * nn * nn + 8.0 * nn * k, 9.0 * nn * nn * nn);
