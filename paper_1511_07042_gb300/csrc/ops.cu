@@ -70,26 +70,31 @@ __device__ __forceinline__ void stv(float* p, size_t i, const float (&v)[4]) {
 // multiply-add in 2.4 (measured).  The row products of float64 blocks are therefore
 // formed in integers, except the first NF nonzeros, which keep the float64 unit busy
 // meanwhile and are added last:
-//   a = A' 2^(Ea - 1081), |A'| < 2^59, Ea the largest exponent field of the row's values;
+//   a = A' 2^(Ea - 1081), |A'| <= 2^59, Ea the largest exponent field of the row's values;
 //   x = X' 2^(Ex - 1082), |X'| < 2^60, Ex the largest one among the row's values of X in
-//   that column; each split into signed 32-bit halves, A' = ah 2^32 + al;
-//   sum a x = (sum ah xh) 2^64 + (sum ah xl + al xh) 2^32, both sums exact in int64 over
-//   kFixNnz nonzeros, and one rounding to nearest at the end.
-// Dropped: al xl and the bits that the alignment shifts out, together below 2^-56 of
-// max|a| max|x| a term.  A float64 sum rounds each of its partial sums at 2^-53.  Against
-// exact sums of 7 products the integer sum's error is at most the float64 sum's (3e-17
-// against 7e-17 of sum |a x| in the mean over Laplacian rows, 5.6e-16 against 5.4e-16 at
-// most over rows of random exponents) where some product of the row comes within
-// kFixSlack bits of max|a| max|x|.  Rows without such a product (large x that all meet
+//   that column; each split into signed parts, A' = ah 2^29 + al, X' = xh 2^30 + xl;
+//   sum a x = (sum ah xh) 2^59 + (sum ah xl + 2 al xh) 2^29, both sums exact in int64 over
+//   kFixNnz nonzeros (below 7 2^60), and one rounding to nearest at the end.
+// The parts are as short as the sums allow (halves of 32 bits would drop a product al xl of
+// 2^62): dropped are al xl (below 2^57), the rounding of A' (half a unit, times |X'| < 2^60) and
+// the bits of X' that the alignment shifts out (a unit, times |A'| <= 2^59), the latter two only
+// where a value is less than 2^-6 (2^-7) of the largest.  A row takes the integer sum where some
+// product comes within kFixSlack bits of max|a| max|x|, so that sum |a x| >= 2^114: the error is
+// then at most 2^-53 |s| + (6 2^59 + 7 2^57 + 2^58) 2^-114 sum |a x| < 3.1 2^-53 sum |a x|,
+// against a bound of 7 2^-53 sum |a x| for a float64 sum of 7 products.  Over rows made for a
+// large error (one product at 2^-3 and the others' small factors with long mantissas) the mean
+// is 3.7e-17 (float64 6.0e-17) and the largest 1.5e-16 (3.6e-16) of sum |a x|, over Laplacian
+// rows 1e-18 to 2e-17 (2.4e-17 to 4e-17).  Rows without such a product (large x that all meet
 // small a), rows longer than kFixNnz, and values outside a band of exponents (zeros among
 // normal values excepted; Inf, NaN and subnormals fall outside) take the float64 loop.
 // Result and error do not depend on the lanes per row.
-// Measured, 655362 x 128: [AX | MX] 1924 -> 1170 us (NF = 2; 1418 and 1350 us with 1 and
-// 3); now bound by the issue of about 55 integer instructions per product pair.
+// Measured, 655362 x 128: [AX | MX] 1924 -> 1121 us (NF = 2; in halves of 32 bits 1169 us,
+// and 1418 and 1350 us with NF = 1 and 3); now bound by the issue of about 55 integer
+// instructions per product pair.
 constexpr int kFixNnz = 7;     // a vertex of a subdivided surface and its six neighbours
 constexpr int kFixSlack = 3;
 struct FixEntry {
-  int ah, al, mh, ml;   // halves of A' and M'
+  int ah, al, mh, ml;   // parts of A' and M' (al, ml doubled)
 };
 struct FixIndex {
   int col, slack;       // column; Ea - ea (low half) and Em - em (high half), at most 0x3fff
@@ -99,21 +104,34 @@ struct FixStage {       // one row of a warp
   FixIndex j[8];
 };
 __device__ __forceinline__ int exp_field(double v) { return (__double2hiint(v) >> 20) & 0x7FF; }
-// v 2^(1081 - emax) (drop = 5) or v 2^(1082 - emax) (drop = 4), rounded towards zero, as
-// h 2^32 + l with a signed l; sh = emax - exponent field of v
-__device__ __forceinline__ void fix_halves(double v, int sh, int drop, int& h, int& l) {
+// the 64 bits of |v| from its leading bit (bit 63) on, shifted right by sh
+__device__ __forceinline__ unsigned long long fix_magnitude(double v, int sh) {
   const int hi = __double2hiint(v), lo = __double2loint(v);
   unsigned long long m = ((unsigned long long)(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | (unsigned)(lo << 11);
-  asm("shr.u64 %0, %1, %2;" : "=l"(m) : "l"(m), "r"(sh + drop));   // a shift past 63 gives 0
-  const long long s = (long long)(hi >> 31);
-  const long long w = ((long long)m ^ s) - s;
-  l = (int)w;
-  h = (int)(w >> 32) - (l >> 31);
+  asm("shr.u64 %0, %1, %2;" : "=l"(m) : "l"(m), "r"(sh));   // a shift past 63 gives 0
+  return m;
 }
-// (hi 2^64 + mid 2^32) 2^(e - 2163): the two sums as one integer in units of 2^-60 of
-// max|a| max|x| (below 2^63: seven products below 2^119, units of 2^59), rounded to nearest
+// A' = v 2^(1081 - emax), rounded to nearest, as ah 2^29 + al2 / 2; sh = emax - exponent field of v
+__device__ __forceinline__ void fix_a(double v, int sh, int& ah, int& al2) {
+  const long long m = (long long)((fix_magnitude(v, sh + 4) + 1) >> 1);
+  const long long w = __double2hiint(v) < 0 ? -m : m;
+  ah = (int)((w + (1ll << 28)) >> 29);
+  al2 = (int)(w - ((long long)ah << 29)) * 2;
+}
+// X' = v 2^(1082 - emax), rounded towards zero, as xh 2^30 + xl.  The sign is applied to the two
+// parts: two 32-bit operations each, where a 64-bit negation before the split let the SpMM take
+// 1380 us (1153 with the split by a bit-field extraction) instead of 1121.
+__device__ __forceinline__ void fix_x(double v, int sh, int& xh, int& xl) {
+  const unsigned long long m = fix_magnitude(v, sh + 4) + (1ull << 29);
+  const int sg = __double2hiint(v) >> 31;
+  xh = ((int)(m >> 30) ^ sg) - sg;
+  xl = (((int)((unsigned)m & 0x3fffffffu) - (1 << 29)) ^ sg) - sg;
+}
+// (hi 2^59 + mid 2^29) 2^(e - 2163): the two sums as one integer in units of 2^59 (kFixMid, the
+// start value of the second sum, rounds it), rounded to nearest
+constexpr long long kFixMid = 1ll << 29;
 __device__ __forceinline__ double fix_value(long long hi, long long mid, int e) {
-  const long long v = (hi << 5) + (mid >> 27);
+  const long long v = hi + (mid >> 30);
   const double d = __ll2double_rn(v);
   return v == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + ((e - 2104) << 20), __double2loint(d));
 }
@@ -160,8 +178,8 @@ __device__ __forceinline__ void gather_row_fixed(const int* __restrict__ col, co
       if (q < NF) {
         f = {__double2hiint(av[t]), __double2loint(av[t]), __double2hiint(mv[t]), __double2loint(mv[t])};
       } else {
-        fix_halves(av[t], ea - xa, 5, f.ah, f.al);
-        fix_halves(mv[t], em - xm, 5, f.mh, f.ml);
+        fix_a(av[t], ea - xa, f.ah, f.al);
+        fix_a(mv[t], em - xm, f.mh, f.ml);
         if (xa == 0) f.ah = f.al = 0;   // zero (all zero or subnormal rows take the other path)
         if (xm == 0) f.mh = f.ml = 0;
       }
@@ -183,7 +201,7 @@ __device__ __forceinline__ void gather_row_fixed(const int* __restrict__ col, co
     for (int z = 0; z < 2; ++z) {
       int ex = 0;
       unsigned best = 0xffffffffu;
-      long long ha = 0, ma = 0, hm = 0, lm = 0;
+      long long ha = 0, ma = kFixMid, hm = 0, lm = kFixMid;
 #pragma unroll
       for (int q = NF; q < kFixNnz; ++q) ex = max(ex, exp_field(x[q][z]));
 #pragma unroll
@@ -191,7 +209,7 @@ __device__ __forceinline__ void gather_row_fixed(const int* __restrict__ col, co
         const FixEntry f = st->e[q];
         const int sh = ex - exp_field(x[q][z]);
         int xh, xl;
-        fix_halves(x[q][z], sh, 4, xh, xl);
+        fix_x(x[q][z], sh, xh, xl);
         best = __vminu2(best, (unsigned)(st->j[q].slack + sh * 0x10001));
         ha += (long long)f.ah * xh;
         ma += (long long)f.ah * xl;
