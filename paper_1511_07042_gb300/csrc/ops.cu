@@ -85,8 +85,8 @@ __device__ __forceinline__ void stv(float* p, size_t i, const float (&v)[4]) {
 // large error (one product at 2^-3 and the others' small factors with long mantissas) the mean
 // is 3.7e-17 (float64 6.0e-17) and the largest 1.5e-16 (3.6e-16) of sum |a x|, over Laplacian
 // rows 1e-18 to 2e-17 (2.4e-17 to 4e-17).  Rows without such a product (large x that all meet
-// small a), rows longer than kFixNnz, and values outside a band of exponents (zeros among
-// normal values excepted; Inf, NaN and subnormals fall outside) take the float64 loop.
+// small a) and values outside a band of exponents (zeros among normal values excepted; Inf, NaN
+// and subnormals fall outside) take a float64 loop, and what a row has beyond kFixNnz too.
 // Result and error do not depend on the lanes per row.
 // Measured, 655362 x 128: [AX | MX] 1924 -> 1121 us (NF = 2; in halves of 32 bits 1169 us,
 // and 1418 and 1350 us with NF = 1 and 3); now bound by the issue of about 55 integer
@@ -143,13 +143,20 @@ __device__ __forceinline__ void gather_row_fixed(const int* __restrict__ col, co
                                                  double (&mm)[CPL][2]) {
   // the row's values as integers, by the first lanes of the row
   constexpr int NQ = LPR >= 8 ? 1 : 8 / LPR;
-  const bool small = len <= kFixNnz && len > NF;
+  // Rows of more than kFixNnz nonzeros: with NF > 0 the first ones take the integer sum and the
+  // others follow one at a time; with NF = 0 (two sums in every kernel, fewer registers left)
+  // the whole row goes one at a time.  A level of random valences, 39994 rows, 8 % of them
+  // longer: [AX | MX] at k = 20 takes 50 us, with whole rows 57, symmetric
+  // Gauss-Seidel with shifts at k = 64 takes 338 us, with the split 372.
+  constexpr bool kSplit = NF > 0;
+  const bool some = len > NF && (kSplit || len <= kFixNnz);   // nonzeros for the integer sum
+  const int cnt = min(len, kFixNnz);
   double av[NQ], mv[NQ];
   int jv[NQ], ea = 0, em = 0;
 #pragma unroll
   for (int t = 0; t < NQ; ++t) {
     const int q = sl + t * LPR;
-    const bool in = small && q < len;
+    const bool in = some && q < cnt;
     jv[t] = in ? __ldcs(col + b + q) : 0;
     av[t] = in ? __ldcs(va + b + q) : 0.0;
     mv[t] = (WITH_M && in) ? __ldcs(vm + b + q) : 0.0;
@@ -185,11 +192,33 @@ __device__ __forceinline__ void gather_row_fixed(const int* __restrict__ col, co
       }
       st->e[q] = f;
       // an absent nonzero reads the row's first column again, with the value 0
-      st->j[q] = {q < len ? jv[t] : j0, (xa ? ea - xa : 0x3fff) | ((xm ? em - xm : 0x3fff) << 16)};
+      st->j[q] = {q < cnt ? jv[t] : j0, (xa ? ea - xa : 0x3fff) | ((xm ? em - xm : 0x3fff) << 16)};
     }
   }
   __syncwarp();
-  const bool row_ok = small && ea >= 130 && ea <= 1900 && (!WITH_M || (em >= 130 && em <= 1900));
+  auto one_by_one = [&](int first) {     // with 16-byte loads
+    for (int p = first; p < b + len; ++p) {
+      const int j = __ldcs(col + p);
+      const double a = __ldcs(va + p), m = WITH_M ? __ldcs(vm + p) : 0.0;
+#pragma unroll
+      for (int u = 0; u < CPL; ++u) {
+        const int c = sl + LPR * u;
+        if (c >= nch) continue;
+        double x[2];
+        ldv_ro(X, (size_t)j * nch + c, x);
+#pragma unroll
+        for (int z = 0; z < 2; ++z) {
+          aa[u][z] = fma(a, x[z], aa[u][z]);
+          if (WITH_M) mm[u][z] = fma(m, x[z], mm[u][z]);
+        }
+      }
+    }
+  };
+  if (!kSplit && !some) {
+    one_by_one(b);
+    return;
+  }
+  const bool row_ok = some && ea >= 130 && ea <= 1900 && (!WITH_M || (em >= 130 && em <= 1900));
 #pragma unroll
   for (int u = 0; u < CPL; ++u) {
     const int c = sl + LPR * u;
@@ -232,13 +261,14 @@ __device__ __forceinline__ void gather_row_fixed(const int* __restrict__ col, co
 #pragma unroll
         for (int q = NF; q < kFixNnz; ++q) zero = zero && x[q][z] == 0.0;
         if (!zero)
-          for (int p = b + (small ? NF : 0); p < b + len; ++p) {
-            const double xv = __ldg(X + ((size_t)col[p] * nch + c) * 2 + z);
-            s = fma(va[p], xv, s);
-            if (WITH_M) t = fma(vm[p], xv, t);
+#pragma unroll 1
+          for (int q = NF; q < cnt; ++q) {
+            const double xv = __ldg(X + ((size_t)st->j[q].col * nch + c) * 2 + z);
+            s = fma(va[b + q], xv, s);
+            if (WITH_M) t = fma(vm[b + q], xv, t);
           }
       }
-      if (small) {
+      if (some) {
 #pragma unroll
         for (int q = 0; q < NF; ++q) {
           const FixEntry f = st->e[q];
@@ -250,6 +280,7 @@ __device__ __forceinline__ void gather_row_fixed(const int* __restrict__ col, co
       if (WITH_M) mm[u][z] = t;
     }
   }
+  if (kSplit) one_by_one(some ? b + kFixNnz : b);
 }
 
 // aa += A_row X, mm += M_row X for one CSR row owned by LPR lanes (pattern and values
