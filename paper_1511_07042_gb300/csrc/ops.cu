@@ -362,10 +362,13 @@ __device__ __forceinline__ void gather_row(const int* __restrict__ col, const T*
 // operations: a conversion between the two costs as much as a float64 operation (64
 // cycles a warp).  Values outside 2^-100 .. 2^100 take the conversions and two Newton steps.
 // FP32: the correctly rounded reciprocal.
+__device__ __forceinline__ bool in_recip_band(double d) {   // 2^-100 <= |d| < 2^100
+  return ((unsigned)__double2hiint(d) & 0x7fffffffu) - 0x39b00000u < 0x46300000u - 0x39b00000u;
+}
 __device__ __forceinline__ double recip(double d) {
   const int hi = __double2hiint(d);
   const unsigned ah = (unsigned)hi & 0x7fffffffu;
-  if (ah - 0x39b00000u < 0x46300000u - 0x39b00000u) {   // 2^-100 <= |d| < 2^100
+  if (in_recip_band(d)) {
     const float f = __uint_as_float(((ah - 0x38000000u) << 3) | ((unsigned)__double2loint(d) >> 29));
     float yf;
     asm("rcp.approx.f32 %0, %1;" : "=f"(yf) : "f"(f));
@@ -380,6 +383,17 @@ __device__ __forceinline__ double recip(double d) {
   return y;
 }
 __device__ __forceinline__ float recip(float d) { return __frcp_rn(d); }
+// num / d.  FP64: from the reciprocal with one correction (a float64 division takes about eight
+// float64 operations) where the reciprocal has its band and the result is finite, else by
+// division: the reciprocal of a larger (smaller) d would be 0 (Inf).
+__device__ __forceinline__ double quotient(double num, double d) {
+  if (in_recip_band(d)) {
+    const double y = recip(d), f = num * y, r = fma(fma(-d, f, num), y, f);
+    if ((~__double2hiint(r) & 0x7FF00000) != 0) return r;
+  }
+  return num / d;
+}
+__device__ __forceinline__ float quotient(float num, float d) { return num / d; }
 
 // ---- fused SpMM: AX = A X, MX = M X  (one pass over the shared pattern) ----
 // Row tiling: LPR lanes per row (32 / LPR rows per warp), CPL 16-byte chunks per lane
@@ -566,9 +580,8 @@ kaczmarz_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col, co
   const int e = live ? row_ptr[row + 1] : 0;
   gather_row<T, LPR, CPL>(col, va, vm, X, b, e - b, nch, sl, st, aa, mm);
   if (!live) return;
-  // ||k_r||^2 = na - 2 s nam + s^2 nm as nested multiply-adds, and the quotient from its
-  // reciprocal with one correction (a float64 division takes about eight float64 operations,
-  // which are what bounds the kernel: 29 -> 24 a value)
+  // ||k_r||^2 = na - 2 s nam + s^2 nm as nested multiply-adds (float64 operations are what
+  // bounds the kernel: 24 a value with this quotient, 29 with a division)
   const T n_a = na[row], n_am2 = T(-2) * nam[row], n_m = nm[row];
   T coef[CPL][W], sv[CPL][W];
 #pragma unroll
@@ -586,8 +599,7 @@ kaczmarz_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col, co
     for (int q = 0; q < W; ++q) {
       const T res = bb[q] - (aa[u][q] - sv[u][q] * mm[u][q]);
       const T nrm = fma(sv[u][q], fma(sv[u][q], n_m, n_am2), n_a);
-      const T num = omega * res, y = recip(nrm), f = num * y;
-      coef[u][q] = nrm > T(0) ? fma(fma(-nrm, f, num), y, f) : T(0);
+      coef[u][q] = nrm > T(0) ? quotient(omega * res, nrm) : T(0);
     }
   }
   for (int p = b; p < e; ++p) {
