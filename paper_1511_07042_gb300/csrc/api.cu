@@ -96,7 +96,7 @@ Workspace::Workspace(size_t bytes, cudaStream_t s) : s_(s) {
   if (!ptr_) {
     bytes_ = (bytes + 0xFFFFF) & ~(size_t)0xFFFFF;   // whole megabytes, so that calls of near sizes share
     cudaError_t e = cudaMalloc(&ptr_, bytes_);
-    if (e != cudaSuccess) {
+    if (e == cudaErrorMemoryAllocation) {
       cudaGetLastError();
       pool_trim();
       e = cudaMalloc(&ptr_, bytes_);
@@ -117,10 +117,12 @@ Workspace::Workspace(size_t bytes, cudaStream_t s) : s_(s) {
 Workspace::~Workspace() {
   if (!ptr_) return;
   if (!idle_) cudaStreamSynchronize(s_);
+  const PoolItem mine{ptr_, bytes_, flag_, dev_};
   std::vector<PoolItem> drop;
-  {
+  try {
     std::lock_guard<std::mutex> lock(g_pool_mu);
-    g_pool.push_back({ptr_, bytes_, flag_, dev_});
+    drop.reserve(g_pool.size() + 1);
+    g_pool.push_back(mine);
     // over the limit: the oldest idle buffers of the device go
     size_t held = 0;
     for (const PoolItem& it : g_pool) held += it.dev == dev_ ? it.bytes : 0;
@@ -130,6 +132,9 @@ Workspace::~Workspace() {
       drop.push_back(g_pool[q]);
       g_pool.erase(g_pool.begin() + q);
     }
+  } catch (...) {        // no host memory: nothing leaves a destructor
+    pool_free(mine);
+    return;
   }
   for (const PoolItem& it : drop) pool_free(it);
 }

@@ -69,7 +69,7 @@ void DBuf<T>::alloc(size_t count) {
   release();
   if (count == 0) return;
   cudaError_t e = cudaMalloc(&ptr, count * sizeof(T));
-  if (e != cudaSuccess) {
+  if (e == cudaErrorMemoryAllocation) {   // (not for a call under capture, which frees nothing)
     cudaGetLastError();
     pool_trim();
     e = cudaMalloc(&ptr, count * sizeof(T));
