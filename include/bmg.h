@@ -23,7 +23,12 @@
  *     `stream` (a cudaStream_t passed as void*; NULL = legacy default stream)
  *     enqueue their work on it and may return before it completes, unless stated.
  *   - Ownership: a bmg_problem owns every device buffer it allocates and frees it
- *     in bmg_destroy.  Buffers passed in by the caller are never freed.
+ *     in bmg_destroy.  Buffers passed in by the caller are never freed.  Beside
+ *     these, the synchronous step calls (bmg_gram, bmg_gram_tc, bmg_expand,
+ *     bmg_dense_eig and their float32 forms) and the set-up take their workspaces from
+ *     a process-wide pool, which keeps at most 64 MB per device between calls.  Every
+ *     bmg_destroy frees what it holds, with NULL too, and so does a device allocation
+ *     of this library that fails for lack of memory.
  *   - Errors: every call returns a bmg_status and never aborts the process.  On an
  *     error the outputs are unspecified (except BMG_ERR_NOT_CONVERGED, see
  *     bmg_solve), and bmg_last_error() returns a message for the calling thread.

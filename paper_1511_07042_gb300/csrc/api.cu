@@ -220,7 +220,6 @@ extern "C" void bmg_default_options(bmg_options* o) {
 extern "C" const char* bmg_last_error(void) { return g_last_error.c_str(); }
 
 extern "C" void bmg_destroy(bmg_problem* p) {
-  if (!p) return;
   try { delete p; } catch (...) {}
   pool_trim();
 }

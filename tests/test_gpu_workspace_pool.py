@@ -42,3 +42,16 @@ def test_failed_call_under_capture_loses_no_buffer(gpu_bmg):
     assert free_bytes() >= before
     gpu_bmg.gram(large, large, 160, G)
     assert torch.equal(G, torch.zeros_like(G))
+
+
+def test_destroying_nothing_empties_the_pool(gpu_bmg):
+    """A program that only calls steps has no problem to destroy."""
+    X = torch.zeros((64, 160), dtype=torch.float64, device="cuda")
+    G = torch.empty((160, 160), dtype=torch.float64, device="cuda")
+    gpu_bmg.gram(X, X, 160, G)
+    gpu_bmg.LIB.bmg_destroy(None)
+    before = free_bytes()
+    gpu_bmg.gram(X, X, 160, G)
+    assert free_bytes() < before
+    gpu_bmg.LIB.bmg_destroy(None)
+    assert free_bytes() >= before
