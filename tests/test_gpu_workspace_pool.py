@@ -17,7 +17,8 @@ def free_bytes():
 
 def test_failed_call_under_capture_loses_no_buffer(gpu_bmg):
     rt = ctypes.CDLL("libcudart.so.13")
-    small, large = (torch.zeros((n, 160), dtype=torch.float64, device="cuda") for n in (64, 160000))
+    # workspaces of 31 and 62 MB (smaller ones come out of memory that the driver keeps anyway)
+    small, large = (torch.zeros((n, 160), dtype=torch.float64, device="cuda") for n in (9600, 20000))
     G = torch.empty((160, 160), dtype=torch.float64, device="cuda")
     stream = torch.cuda.Stream()
 
@@ -46,7 +47,7 @@ def test_failed_call_under_capture_loses_no_buffer(gpu_bmg):
 
 def test_destroying_nothing_empties_the_pool(gpu_bmg):
     """A program that only calls steps has no problem to destroy."""
-    X = torch.zeros((64, 160), dtype=torch.float64, device="cuda")
+    X = torch.zeros((9600, 160), dtype=torch.float64, device="cuda")
     G = torch.empty((160, 160), dtype=torch.float64, device="cuda")
     gpu_bmg.gram(X, X, 160, G)
     gpu_bmg.LIB.bmg_destroy(None)
