@@ -340,6 +340,9 @@ size_t expand_tc_scratch_bytes(int k);
 template <typename TI>
 void gram_tc(const TI* X, const TI* Y, int n, int k, int ld, double* G, double* partial, int nparts, int* err,
              cudaStream_t s, bool sym);
+// columns c0 .. ld - 1 of U: those of Zf, or zero without it
+template <typename T>
+void expand_pad(const T* Zf, int n, int c0, int ld, T* U, cudaStream_t s);
 template <typename TI>
 void expand_tc(const TI* Zf, const TI* X, const double* Yx, int n, int k, int ld, int ldy, TI* U,
                unsigned char* scratch, int* err, cudaStream_t s);

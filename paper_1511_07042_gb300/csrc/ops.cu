@@ -950,6 +950,15 @@ __global__ void eigres_kernel(const T* __restrict__ AU, const T* __restrict__ MU
 }
 
 // ---- expand: U = Zf + X Yx ----------------------------------------------------
+// Columns c0 .. ld - 1 of U: those of Z, or zero (paddings wider than the columns that the
+// expansion kernels write).
+template <typename T>
+__global__ void expand_pad_kernel(const T* Z, int n, int c0, int ld, T* U) {
+  const int c = c0 + blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= ld) return;
+  for (int r = blockIdx.y; r < n; r += gridDim.y) U[(size_t)r * ld + c] = Z ? Z[(size_t)r * ld + c] : T(0);
+}
+
 // One warp per row; Yx (k x ldy, FP64) staged in shared memory as T; lane owns the
 // chunks lane + 32 u of the output row.
 template <typename T, int CPL>
@@ -1430,6 +1439,15 @@ void eig_residuals(const T* AU, const T* MU, const T* U, const double* lam, int 
 }
 
 template <typename T>
+void expand_pad(const T* Zf, int n, int c0, int ld, T* U, cudaStream_t s) {
+  if (c0 >= ld) return;
+  expand_pad_kernel<T><<<dim3((ld - c0 + 127) / 128, std::min(n, 16384)), 128, 0, s>>>(Zf, n, c0, ld, U);
+  check_launch("expand_pad_kernel");
+}
+template void expand_pad<double>(const double*, int, int, int, double*, cudaStream_t);
+template void expand_pad<float>(const float*, int, int, int, float*, cudaStream_t);
+
+template <typename T>
 void expand(const T* Zf, const T* X, const double* Yx, int n, int k, int ld, int ldy, T* U,
             cudaStream_t s) {
   const int nch = ld / Chunk<T>::W;
@@ -1448,6 +1466,7 @@ void expand(const T* Zf, const T* X, const double* Yx, int n, int k, int ld, int
       expand_kernel<T, 4><<<grid, kWarpsPerBlock * 32, smem, s>>>(Zf, X, Yx, n, k, ld, ldy, U); break;
   }
   check_launch("expand_kernel");
+  expand_pad(Zf, n, 128 * Chunk<T>::W, ld, U, s);   // the kernel takes at most 128 chunks of a row
   prof_end(KC_EXPAND, s, 3.0 * tb<T>() * n * ld + 8.0 * k * k, 2.0 * n * k * k);
 }
 

@@ -1230,6 +1230,7 @@ void expand_tc_launch(const TI* Zf, const TI* X, const double* Yx, int n, int k,
   check_launch("expand_prep_kernel");
   expand_tc_kernel<TI><<<grid, kTcThreads, smem, s>>>(Zf, X, scratch, gexp, n, k, ld, nsub, njb, U, vec, err, ctl);
   check_launch("expand_tc_kernel");
+  expand_pad(Zf, n, njb * kNB, ld, U, s);
   prof_end(KC_EXPAND, s, 3.0 * sizeof(TI) * n * ld + 8.0 * k * k, 2.0 * n * k * k);
 }
 }  // namespace
