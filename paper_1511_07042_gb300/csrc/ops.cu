@@ -64,6 +64,15 @@ __device__ __forceinline__ void stv(float* p, size_t i, const float (&v)[4]) {
   reinterpret_cast<float4*>(p)[i] = make_float4(v[0], v[1], v[2], v[3]);
 }
 
+// First chunk of lane sl of a row.  The widest shape (32 lanes of 4 chunks) takes 128 chunks of a
+// row, blockIdx.y the slab of them, so that rows of any length are covered.
+constexpr int kSlab = 128;
+template <int CPL>
+__device__ __forceinline__ int first_chunk(int sl) {
+  return CPL == 4 ? sl + kSlab * (int)blockIdx.y : sl;
+}
+inline unsigned slabs(int cpl, int nch) { return cpl == 4 ? (unsigned)((nch + kSlab - 1) / kSlab) : 1u; }
+
 // ---- float64 rows in integer arithmetic ---------------------------------------
 // GB300 retires a float64 multiply-add per warp and scheduler every 64 cycles, an
 // integer add every one, a shift or logic operation every two and a 32 x 32 + 64
@@ -139,7 +148,7 @@ __device__ __forceinline__ double fix_value(long long hi, long long mid, int e) 
 template <int LPR, int CPL, bool WITH_M, int NF>
 __device__ __forceinline__ void gather_row_fixed(const int* __restrict__ col, const double* __restrict__ va,
                                                  const double* __restrict__ vm, const double* __restrict__ X, int b,
-                                                 int len, int nch, int sl, FixStage* st, double (&aa)[CPL][2],
+                                                 int len, int nch, int sl, int cl, FixStage* st, double (&aa)[CPL][2],
                                                  double (&mm)[CPL][2]) {
   // the row's values as integers, by the first lanes of the row
   constexpr int NQ = LPR >= 8 ? 1 : 8 / LPR;
@@ -202,7 +211,7 @@ __device__ __forceinline__ void gather_row_fixed(const int* __restrict__ col, co
       const double a = __ldcs(va + p), m = WITH_M ? __ldcs(vm + p) : 0.0;
 #pragma unroll
       for (int u = 0; u < CPL; ++u) {
-        const int c = sl + LPR * u;
+        const int c = cl + LPR * u;
         if (c >= nch) continue;
         double x[2];
         ldv_ro(X, (size_t)j * nch + c, x);
@@ -221,7 +230,7 @@ __device__ __forceinline__ void gather_row_fixed(const int* __restrict__ col, co
   const bool row_ok = some && ea >= 130 && ea <= 1900 && (!WITH_M || (em >= 130 && em <= 1900));
 #pragma unroll
   for (int u = 0; u < CPL; ++u) {
-    const int c = sl + LPR * u;
+    const int c = cl + LPR * u;
     if (c >= nch) continue;
     double x[kFixNnz][2];
 #pragma unroll
@@ -302,12 +311,12 @@ struct GatherWidth {
 template <typename T, int LPR, int CPL, bool WITH_M = true, int NF = 0>
 __device__ __forceinline__ void gather_row(const int* __restrict__ col, const T* __restrict__ va,
                                            const T* __restrict__ vm, const T* __restrict__ X, int b, int len,
-                                           int nch, int sl, FixStage* st, T (&aa)[CPL][Chunk<T>::W],
+                                           int nch, int sl, int cl, FixStage* st, T (&aa)[CPL][Chunk<T>::W],
                                            T (&mm)[CPL][Chunk<T>::W]) {
   // WITH_M = false: only A x (mm untouched), for shifted problems with shift 0
   constexpr int W = Chunk<T>::W;
   if constexpr (sizeof(T) == 8) {
-    gather_row_fixed<LPR, CPL, WITH_M, NF>(col, va, vm, X, b, len, nch, sl, st, aa, mm);
+    gather_row_fixed<LPR, CPL, WITH_M, NF>(col, va, vm, X, b, len, nch, sl, cl, st, aa, mm);
     return;
   } else {
   constexpr int G = GatherWidth<T, LPR, CPL>::G;
@@ -327,7 +336,7 @@ __device__ __forceinline__ void gather_row(const int* __restrict__ col, const T*
       const int j = __shfl_sync(0xffffffffu, jl, q, LPR);
 #pragma unroll
       for (int u = 0; u < CPL; ++u) {
-        const int c = sl + LPR * u;
+        const int c = cl + LPR * u;
         if (q < cnt && c < nch) {
           ldv_ro(X, (size_t)j * nch + c, x[q][u]);
         } else {
@@ -343,7 +352,7 @@ __device__ __forceinline__ void gather_row(const int* __restrict__ col, const T*
       if (q < cnt) {
 #pragma unroll
         for (int u = 0; u < CPL; ++u)
-          if (sl + LPR * u < nch) {
+          if (cl + LPR * u < nch) {
 #pragma unroll
             for (int z = 0; z < W; ++z) {
               aa[u][z] = fma(a, x[q][u][z], aa[u][z]);
@@ -420,7 +429,7 @@ spmm_am_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
   constexpr int RPW = 32 / LPR;
   __shared__ FixStage stage[sizeof(T) == 8 ? 8 * RPW : 1];   // float64 blocks: a row of each warp part
   FixStage* st = stage + (sizeof(T) == 8 ? (threadIdx.x >> 5) * RPW + (threadIdx.x & 31) / LPR : 0);
-  const int lane = threadIdx.x & 31, sl = lane % LPR;
+  const int lane = threadIdx.x & 31, sl = lane % LPR, cl = first_chunk<CPL>(sl);
   const int per_group = (blockDim.x >> 5) * RPW;
   const int ngroups = (n + per_group - 1) / per_group;
   const int w0 = (threadIdx.x >> 5) * RPW + lane / LPR;
@@ -440,11 +449,11 @@ spmm_am_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
 #pragma unroll
       for (int q = 0; q < W; ++q) { aa[u][q] = T(0); mm[u][q] = T(0); }
     const int b = live ? row_ptr[row] : 0;
-    gather_row<T, LPR, CPL, true, 2>(col, va, vm, X, b, live ? row_ptr[row + 1] - b : 0, nch, sl, st, aa, mm);
+    gather_row<T, LPR, CPL, true, 2>(col, va, vm, X, b, live ? row_ptr[row + 1] - b : 0, nch, sl, cl, st, aa, mm);
     if (!live) continue;
 #pragma unroll
     for (int u = 0; u < CPL; ++u) {
-      const int c = sl + LPR * u;
+      const int c = cl + LPR * u;
       if (c < nch) {
         stv_cs(AX, (size_t)row * nch + c, aa[u]);
         stv_cs(MX, (size_t)row * nch + c, mm[u]);
@@ -481,7 +490,7 @@ row_update_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
   constexpr int RPW = 32 / LPR;
   __shared__ FixStage stage[sizeof(T) == 8 ? 8 * RPW : 1];   // float64 blocks: a row of each warp part
   FixStage* st = stage + (sizeof(T) == 8 ? (threadIdx.x >> 5) * RPW + (threadIdx.x & 31) / LPR : 0);
-  const int lane = threadIdx.x & 31, sl = lane % LPR;
+  const int lane = threadIdx.x & 31, sl = lane % LPR, cl = first_chunk<CPL>(sl);
   const int per_group = (blockDim.x >> 5) * RPW;
   const int ngroups = (nrows + per_group - 1) / per_group;
   constexpr bool kNext = sizeof(T) == 4 || !ZS;
@@ -510,15 +519,15 @@ row_update_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
     for (int u = 0; u < CPL; ++u) {
 #pragma unroll
       for (int q = 0; q < W; ++q) bb[u][q] = T(0);
-      if (kAhead && B && live && sl + LPR * u < nch) ldv(B, (size_t)row * nch + sl + LPR * u, bb[u]);
+      if (kAhead && B && live && cl + LPR * u < nch) ldv(B, (size_t)row * nch + cl + LPR * u, bb[u]);
     }
     const T dai = live ? __ldg(da + row) : T(0), dmi = (ZS || !live) ? T(0) : __ldg(dm + row);
-    gather_row<T, LPR, CPL, !ZS, ZS ? 2 : 0>(col, va, vm, X, b, live ? row_ptr[row + 1] - b : 0, nch, sl, st, aa, mm);
+    gather_row<T, LPR, CPL, !ZS, ZS ? 2 : 0>(col, va, vm, X, b, live ? row_ptr[row + 1] - b : 0, nch, sl, cl, st, aa, mm);
     if (!live) continue;
     const T rd0 = (ZS && MODE != 2) ? recip(dai) : T(0);
 #pragma unroll
     for (int u = 0; u < CPL; ++u) {
-      const int c = sl + LPR * u;
+      const int c = cl + LPR * u;
       if (c >= nch) continue;
       T s[W], r[W];
       if (ZS) {
@@ -567,7 +576,7 @@ kaczmarz_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col, co
   constexpr int RPW = 32 / LPR;
   __shared__ FixStage stage[sizeof(T) == 8 ? 8 * RPW : 1];   // float64 blocks: a row of each warp part
   FixStage* st = stage + (sizeof(T) == 8 ? (threadIdx.x >> 5) * RPW + (threadIdx.x & 31) / LPR : 0);
-  const int lane = threadIdx.x & 31, sl = lane % LPR;
+  const int lane = threadIdx.x & 31, sl = lane % LPR, cl = first_chunk<CPL>(sl);
   const int w = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * RPW + lane / LPR;
   const bool live = w < nrows;
   const int row = live ? rows[w] : 0;
@@ -578,7 +587,7 @@ kaczmarz_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col, co
     for (int q = 0; q < W; ++q) { aa[u][q] = T(0); mm[u][q] = T(0); }
   const int b = live ? row_ptr[row] : 0;
   const int e = live ? row_ptr[row + 1] : 0;
-  gather_row<T, LPR, CPL>(col, va, vm, X, b, e - b, nch, sl, st, aa, mm);
+  gather_row<T, LPR, CPL>(col, va, vm, X, b, e - b, nch, sl, cl, st, aa, mm);
   if (!live) return;
   // ||k_r||^2 = na - 2 s nam + s^2 nm as nested multiply-adds (float64 operations are what
   // bounds the kernel: 24 a value with this quotient, 29 with a division)
@@ -586,7 +595,7 @@ kaczmarz_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col, co
   T coef[CPL][W], sv[CPL][W];
 #pragma unroll
   for (int u = 0; u < CPL; ++u) {
-    const int c = sl + LPR * u;
+    const int c = cl + LPR * u;
 #pragma unroll
     for (int q = 0; q < W; ++q) { coef[u][q] = T(0); sv[u][q] = T(0); }
     if (c >= nch) continue;
@@ -607,7 +616,7 @@ kaczmarz_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col, co
     const T a = va[p], m = vm[p];
 #pragma unroll
     for (int u = 0; u < CPL; ++u) {
-      const int c = sl + LPR * u;
+      const int c = cl + LPR * u;
       if (c < nch) {
         T x[W];
         ldv(X, (size_t)j * nch + c, x);
@@ -1091,8 +1100,8 @@ void spmm_shape(int wpb, int chunk, const Mesh& m, const T* a, const T* mm, cons
   int grid, groups;
   row_grid((const void*)spmm_am_kernel<T, LPR, CPL>, wpb * 32, blocks_for(m.n, per_block), per_block, chunk, grid,
            groups);
-  spmm_am_kernel<T, LPR, CPL><<<grid, wpb * 32, 0, s>>>(m.row_ptr.get(), m.col.get(), a, mm, X, m.n, nch, AX, MX,
-                                                        m.row_order.get(), groups);
+  spmm_am_kernel<T, LPR, CPL><<<dim3(grid, slabs(CPL, nch)), wpb * 32, 0, s>>>(
+      m.row_ptr.get(), m.col.get(), a, mm, X, m.n, nch, AX, MX, m.row_order.get(), groups);
   check_launch("spmm_am_kernel");
 }
 template <typename T>
@@ -1117,8 +1126,8 @@ void row_shape(int wpb, int chunk, const Mesh& m, const T* a, const T* mm, const
   int grid, groups;
   row_grid((const void*)row_update_kernel<T, LPR, CPL, MODE, ZS>, wpb * 32, blocks_for(nrows, per_block), per_block,
            chunk, grid, groups);
-  row_update_kernel<T, LPR, CPL, MODE, ZS><<<grid, wpb * 32, 0, s>>>(m.row_ptr.get(), m.col.get(), a, mm, da, dm, rows,
-                                                                 nrows, X, Out, B, shift, nch, (T)omega, groups);
+  row_update_kernel<T, LPR, CPL, MODE, ZS><<<dim3(grid, slabs(CPL, nch)), wpb * 32, 0, s>>>(
+      m.row_ptr.get(), m.col.get(), a, mm, da, dm, rows, nrows, X, Out, B, shift, nch, (T)omega, groups);
   check_launch("row_update_kernel");
 }
 template <typename T, int MODE, bool ZS>
@@ -1299,8 +1308,8 @@ void kaczmarz_colour_sweep(const Mesh& m, const Level& lv, int c, const T* a, co
     kaczmarz_kernel<T, 32, 2><<<blocks_for(nrows, wpb), wpb * 32, 0, s>>>(m.row_ptr.get(), m.col.get(), a, mm, na, nam,
                                                                           nm, rows, nrows, X, B, shift, nch, (T)omega);
   else
-    kaczmarz_kernel<T, 32, 4><<<blocks_for(nrows, wpb), wpb * 32, 0, s>>>(m.row_ptr.get(), m.col.get(), a, mm, na, nam,
-                                                                          nm, rows, nrows, X, B, shift, nch, (T)omega);
+    kaczmarz_kernel<T, 32, 4><<<dim3(blocks_for(nrows, wpb), slabs(4, nch)), wpb * 32, 0, s>>>(
+        m.row_ptr.get(), m.col.get(), a, mm, na, nam, nm, rows, nrows, X, B, shift, nch, (T)omega);
   check_launch("kaczmarz_kernel");
   const double nnz = (double)lv.col2.nnz_host[c];
   // matrix rows, norms, own-row b, gathered block and the written neighbour rows
