@@ -18,7 +18,9 @@
 //   3. FP32 start: eig32_cl_kernel [8-CTA cluster] Householder tridiagonalisation of
 //      sym(T) and multisection on Sturm counts for all eigenvalues; invit_kernel [one CTA per
 //      cluster] inverse iteration with Gram-Schmidt inside clusters of close
-//      eigenvalues; backtr_kernel [multi-CTA] the back-transformation.
+//      eigenvalues; backtr_kernel [multi-CTA] the back-transformation.  (Where the callers
+//      repeat a solve whose refinement did not converge, the last attempt starts from
+//      jacobi_start_kernel instead.)
 //   4. refinement      [multi-CTA, FP64]  the eigenvectors W are refined to FP64
 //      accuracy by the iterative scheme of Ogita & Aishima (2018):
 //          G = W^T W, R = I - G, S = W^T T W, lt_i = s_ii / (1 - r_ii),

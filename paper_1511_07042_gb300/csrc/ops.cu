@@ -477,7 +477,8 @@ spmm_am_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
 // (-> 594 with the launch bound of the product above);
 // 40962 x 64 float64 symmetric Gauss-Seidel with shifts 226 -> 225 -> 221; the float64 sweeps
 // of a 655362-vertex solve at zero shift take 41.3 to 42.2 ms with B ahead, 42.6 with the
-// number, 42.2 with neither.  The product above: 1190 -> 1170 us in float64.
+// number, 42.2 with neither.  The product above: 1190 -> 1170 us in float64 (all in halves of 32
+// bits, see above).
 template <typename T, int LPR, int CPL, int MODE, bool ZS>
 __global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512, sizeof(T) == 8 ? 3 : 0)
 row_update_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col,
@@ -650,8 +651,10 @@ __global__ void row_norms_kernel(const int* __restrict__ row_ptr, const T* __res
 // gathers (row order, then parents; row order, row extent, then midpoints) is hidden by the
 // number of threads: warps that take rows in turn with the chain run ahead were slower
 // (655362 x 128 float64, restriction and added prolongation: 854 us).
-// What bounds the float64 form is the float64 unit (85 % busy): an addition and a
-// multiply-add a value of an added prolongation, six multiply-adds a value of a restriction.
+// What bounds the float64 form is the float64 unit (its pipe is 85 % busy in the added
+// prolongation, 81 % in the restriction, at 163842 x 128): an addition and a multiply-add a
+// value of an added prolongation, seven multiply-adds issued a value of a restriction.  At 64
+// cycles a warp's operation these take 633 us of the 752 us at 655362 x 128.
 // half_of(v) = v / 2 exactly: a float64 product holds the float64 unit for 64 cycles a
 // warp, which is most of what these kernels compute, so the exponent is lowered instead.
 __device__ __forceinline__ float half_of(float v) { return 0.5f * v; }
