@@ -17,7 +17,7 @@ def free_bytes():
 
 def test_failed_call_under_capture_loses_no_buffer(gpu_bmg):
     rt = ctypes.CDLL("libcudart.so.13")
-    # workspaces of 31 and 62 MB (smaller ones come out of memory that the driver keeps anyway)
+    # workspaces of 31 and 62 MB (smaller ones do not change the free bytes that CUDA reports)
     small, large = (torch.zeros((n, 160), dtype=torch.float64, device="cuda") for n in (9600, 20000))
     G = torch.empty((160, 160), dtype=torch.float64, device="cuda")
     stream = torch.cuda.Stream()
